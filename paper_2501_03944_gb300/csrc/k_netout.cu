@@ -8,7 +8,8 @@
 // contiguous chunks of i, each a chain of fmaf in index order, the chunk sums
 // added in chunk order, then the bias), so a spark's fitness does not depend
 // on which sparks share the launch.  The last layer writes the fitness.  An
-// FP64 forward of one vector gives the reported best fitness.
+// FP64 forward of one vector (a launch per layer) gives the reported best
+// fitness.
 #include "mgfwa_internal.cuh"
 
 namespace mgfwa {
@@ -170,35 +171,37 @@ __global__ void __launch_bounds__(256, TR == 4 ? 4 : 2) k_net_layer(const float*
   }
 }
 
-// FP64 forward of one vector (one block): each layer's outputs in parallel,
-// each a dot product in index order, activations in shared memory.
-__global__ void __launch_bounds__(256) k_net_f64(NetOut net, const float* __restrict__ x, double* __restrict__ out) {
+// One layer of the FP64 forward of one vector: one warp per output, lanes
+// striding over the fan-in in index order (coalesced weight reads), then a
+// fixed xor tree and the bias.  `xin` is the FP32 vector for the first layer,
+// `ain` the previous layer's FP64 outputs otherwise.  The layer's weights are
+// read once by as many SMs as it has warps; one block reading every row
+// through its own threads, uncoalesced, was one SM's latency-bound chain
+// (1,882 us for the 1000-512x11-1 network, 12 such launches 60 us).
+constexpr int kF64Warps = 4;
+
+__global__ void __launch_bounds__(32 * kF64Warps) k_net_f64_layer(const float* __restrict__ W,
+                                                                  const float* __restrict__ bias, int32_t fi,
+                                                                  int32_t fo, int32_t act,
+                                                                  const float* __restrict__ xin,
+                                                                  const double* __restrict__ ain,
+                                                                  double* __restrict__ out) {
+  const int j = blockIdx.x * kF64Warps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   griddep_wait();
   griddep_launch_dependents();
-  extern __shared__ double sh[];
-  double* a = sh;
-  double* b = sh + net.wmax;
-  for (int i = threadIdx.x; i < net.widths[0]; i += blockDim.x) a[i] = (double)x[i];
-  __syncthreads();
-  for (int l = 0; l < net.n_layers; ++l) {
-    const int fi = net.widths[l], fo = net.widths[l + 1];
-    const float* W = net.params + net.w_off[l];
-    const float* bias = net.params + net.b_off[l];
-    for (int j = threadIdx.x; j < fo; j += blockDim.x) {
-      double s = (double)bias[j];
-      for (int i = 0; i < fi; ++i) s += (double)W[(int64_t)j * fi + i] * a[i];
-      if (l + 1 < net.n_layers) {
-        const int ak = net.acts[l];
-        s = ak == kActTanh ? tanh(s) : (ak == kActGelu ? 0.5 * s * (1.0 + erf(s * 0.70710678118654752440)) : fmax(s, 0.0));
-      }
-      b[j] = s;
-    }
-    __syncthreads();
-    double* t = a;
-    a = b;
-    b = t;
-  }
-  if (threadIdx.x == 0) *out = a[0];
+  if (j >= fo) return;
+  const float* w = W + (int64_t)j * fi;
+  double s = 0.0;
+#pragma unroll 8
+  for (int i = lane; i < fi; i += 32) s += (double)w[i] * (xin != nullptr ? (double)xin[i] : ain[i]);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if (lane != 0) return;
+  s += (double)bias[j];
+  if (act >= 0)
+    s = act == kActTanh ? tanh(s)
+                        : (act == kActGelu ? 0.5 * s * (1.0 + erf(s * 0.70710678118654752440)) : fmax(s, 0.0));
+  out[j] = s;
 }
 
 }  // namespace
@@ -245,10 +248,19 @@ int launch_net_output(const NetOut& net, const float* rows, int64_t ld, int32_t 
   return n;
 }
 
-int launch_net_output_f64(const NetOut& net, const float* x, double* out, cudaStream_t s) {
-  const size_t smem = sizeof(double) * 2 * (size_t)net.wmax;
-  if (smem > 48 * 1024 && ensure_smem_limit<k_net_f64>(smem) != cudaSuccess) return -1;
-  return launch_pdl(k_net_f64, dim3(1), dim3(256), smem, s, net, x, out) == cudaSuccess ? 1 : -1;
+int launch_net_output_f64(const NetOut& net, const float* x, double* scratch, double* out, cudaStream_t s) {
+  const double* in = nullptr;
+  for (int l = 0; l < net.n_layers; ++l) {
+    const int fi = net.widths[l], fo = net.widths[l + 1];
+    const bool last = l + 1 == net.n_layers;
+    double* o = last ? out : scratch + (int64_t)(l & 1) * net.wmax;
+    if (launch_pdl(k_net_f64_layer, dim3((unsigned)((fo + kF64Warps - 1) / kF64Warps)), dim3(32 * kF64Warps), 0, s,
+                   net.params + net.w_off[l], net.params + net.b_off[l], fi, fo, last ? -1 : net.acts[l],
+                   l == 0 ? x : (const float*)nullptr, in, o) != cudaSuccess)
+      return -1;
+    in = o;
+  }
+  return net.n_layers;
 }
 
 }  // namespace mgfwa

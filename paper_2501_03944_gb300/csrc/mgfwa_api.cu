@@ -885,7 +885,8 @@ size_t carve_all(mgfwa_t* h, char* base) {
   }
   h->best_x = carve<float>(cur, (int64_t)p.B * p.Dp);
   h->best_f = carve<float>(cur, p.B);
-  h->ce64 = carve<double>(cur, N > 0 ? N : 1);
+  // FP64 evaluation of one vector: the batch's losses, or the testbed network's layer outputs (two layers in turn)
+  h->ce64 = carve<double>(cur, h->kind == MGFWA_OBJ_NET_OUTPUT ? 2 * h->net.wmax : (N > 0 ? N : 1));
   h->f64 = carve<double>(cur, 1);
   h->status = carve<uint32_t>(cur, 1);
   h->gens_done = carve<uint32_t>(cur, 1);
@@ -1109,7 +1110,7 @@ mgfwa_status mgfwa_best_run(mgfwa_t* h, int32_t run, float* x_out, double* f_out
     if (h->kind == MGFWA_OBJ_SPHERE)
       MG_LAUNCH(h, launch_sphere_f64(bx, h->p.D, h->f64, h->stream), "FP64 sphere");
     else if (h->kind == MGFWA_OBJ_NET_OUTPUT)
-      MG_LAUNCH(h, launch_net_output_f64(h->net, bx, h->f64, h->stream), "FP64 network output");
+      MG_LAUNCH(h, launch_net_output_f64(h->net, bx, h->ce64, h->f64, h->stream), "FP64 network output");
     else
       MG_LAUNCH(h, launch_fitness_f64(h->mlp, bx, h->ce64, h->f64, h->stream), "FP64 fitness");
     if (cudaMemcpyAsync(f_out, h->f64, sizeof(double), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess)
