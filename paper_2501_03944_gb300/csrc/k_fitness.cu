@@ -148,44 +148,19 @@ __global__ void __launch_bounds__(kThreads) k_fitness_simt(Mlp mlp, const float*
 }
 
 // Small two-layer networks (d_in = DI, h1 = H1, C classes, all compile-time):
-// one block = 128 samples (one per thread, its inputs in registers) x up to
-// kSmallSparks sparks, whose rows are staged in shared memory and read as
-// broadcasts.  Each hidden unit is accumulated over the inputs in ascending
-// order from zero, then the bias is added and the activation applied, and
-// each logit starts from its bias and accumulates the hidden units in
-// ascending order: the same operations in the same order as k_fitness_simt,
-// so both kernels give bitwise the same fitness.  The block's cross-entropy
-// sum per spark goes to partial[mt][row] (warp sums added in warp order, as
-// there).
-constexpr int kSmallSparks = 8;
-
+// one thread = one sample (its inputs in registers) of one spark, whose row is
+// staged in shared memory and read as broadcasts.  Each hidden unit is
+// accumulated over the inputs in ascending order from zero, then the bias is
+// added and the activation applied, and each logit starts from its bias and
+// accumulates the hidden units in ascending order: the same operations in the
+// same order as k_fitness_simt, so every kernel here gives bitwise the same
+// fitness.
 template <int DI, int H1, int C>
-__global__ void __launch_bounds__(kMT) k_fitness_small(Mlp mlp, const float* __restrict__ rows, int64_t ld,
-                                                       int32_t count, const int32_t* __restrict__ idx,
-                                                       float* __restrict__ partial) {
-  constexpr int D = DI * H1 + H1 + C * H1 + C;   // parameters per spark (nn.Linear order)
-  constexpr int kB1 = DI * H1, kW2 = kB1 + H1, kB2 = kW2 + C * H1;
-  __shared__ float ws[kSmallSparks][D];
-  __shared__ float red[kSmallSparks][kMT / 32];
-  griddep_wait();
-  griddep_launch_dependents();
-  const int s0 = blockIdx.x * kSmallSparks, mt = blockIdx.y;
-  const int gs = min(kSmallSparks, count - s0);
-  for (int e = threadIdx.x; e < gs * D; e += kMT) {
-    const int g = e / D, k = e - g * D;
-    const int r = s0 + g;
-    ws[g][k] = rows[(int64_t)(idx != nullptr ? idx[r] : r) * ld + k];
-  }
-  const int64_t n = (int64_t)mt * kMT + threadIdx.x;
-  const bool valid = n < mlp.N;
-  float x[DI];
-#pragma unroll
-  for (int i = 0; i < DI; ++i) x[i] = valid ? mlp.X[n * DI + i] : 0.0f;
-  const int label = valid ? mlp.y[n] : 0;
-  const int act = mlp.acts[0];
-  __syncthreads();
-  for (int g = 0; g < gs; ++g) {
-    const float* W = ws[g];
+struct SmallNet {
+  static constexpr int D = DI * H1 + H1 + C * H1 + C;  // parameters per spark (nn.Linear order)
+  static constexpr int kB1 = DI * H1, kW2 = kB1 + H1, kB2 = kW2 + C * H1;
+  // cross-entropy of one sample
+  static __device__ __forceinline__ float ce(const float* W, const float* x, int label, int act) {
     float z[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) z[c] = W[kB2 + c];
@@ -198,19 +173,54 @@ __global__ void __launch_bounds__(kMT) k_fitness_small(Mlp mlp, const float* __r
 #pragma unroll
       for (int c = 0; c < C; ++c) z[c] = fmaf(W[kW2 + c * H1 + j], a, z[c]);
     }
-    float ce = 0.0f;
-    if (valid) {
-      float zmax = z[0];
+    float zmax = z[0];
 #pragma unroll
-      for (int c = 1; c < C; ++c) zmax = fmaxf(zmax, z[c]);
-      float se = 0.0f;
+    for (int c = 1; c < C; ++c) zmax = fmaxf(zmax, z[c]);
+    float se = 0.0f;
 #pragma unroll
-      for (int c = 0; c < C; ++c) se += expf(z[c] - zmax);
-      float zy = z[0];
+    for (int c = 0; c < C; ++c) se += expf(z[c] - zmax);
+    float zy = z[0];
 #pragma unroll
-      for (int c = 1; c < C; ++c) zy = label == c ? z[c] : zy;
-      ce = (zmax + logf(se)) - zy;
-    }
+    for (int c = 1; c < C; ++c) zy = label == c ? z[c] : zy;
+    return (zmax + logf(se)) - zy;
+  }
+};
+
+// One block = 128 samples x up to `per` sparks, one after another; the
+// block's cross-entropy sum per spark goes to partial[mt][row] (warp sums
+// added in warp order, as in k_fitness_simt).  What bounds a small launch is
+// the chain of one spark's 16 activations times the sparks a block takes in
+// turn, so the launcher gives each block one spark until the blocks fill the
+// GPU (200 and 20 sparks x 512 samples with eight per block: 14.3 us a
+// launch either way; with one, whole generations went from 91 to 30 us).
+constexpr int kSmallSparks = 8;
+
+template <int DI, int H1, int C>
+__global__ void __launch_bounds__(kMT) k_fitness_small(Mlp mlp, const float* __restrict__ rows, int64_t ld,
+                                                       int32_t count, int32_t per, const int32_t* __restrict__ idx,
+                                                       float* __restrict__ partial) {
+  using Net = SmallNet<DI, H1, C>;
+  __shared__ float ws[kSmallSparks][Net::D];
+  __shared__ float red[kSmallSparks][kMT / 32];
+  griddep_wait();
+  griddep_launch_dependents();
+  const int s0 = blockIdx.x * per, mt = blockIdx.y;
+  const int gs = min(per, count - s0);
+  for (int e = threadIdx.x; e < gs * Net::D; e += kMT) {
+    const int g = e / Net::D, k = e - g * Net::D;
+    const int r = s0 + g;
+    ws[g][k] = rows[(int64_t)(idx != nullptr ? idx[r] : r) * ld + k];
+  }
+  const int64_t n = (int64_t)mt * kMT + threadIdx.x;
+  const bool valid = n < mlp.N;
+  float x[DI];
+#pragma unroll
+  for (int i = 0; i < DI; ++i) x[i] = valid ? mlp.X[n * DI + i] : 0.0f;
+  const int label = valid ? mlp.y[n] : 0;
+  const int act = mlp.acts[0];
+  __syncthreads();
+  for (int g = 0; g < gs; ++g) {
+    float ce = valid ? Net::ce(ws[g], x, label, act) : 0.0f;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ce += __shfl_xor_sync(0xffffffffu, ce, off);
     if ((threadIdx.x & 31) == 0) red[g][threadIdx.x >> 5] = ce;
@@ -372,9 +382,12 @@ int launch_fitness_simt_main(const Mlp& mlp, const float* rows, int64_t ld, int3
   if (count <= 0) return 0;
   const int mtiles = (int)((mlp.N + kMT - 1) / kMT);
   if (small_net(mlp, 8, 16, 3)) {
-    dim3 grid((count + kSmallSparks - 1) / kSmallSparks, mtiles);
-    return launch_pdl(k_fitness_small<8, 16, 3>, grid, dim3(kMT), 0, s, mlp, rows, ld, count, idx, partial) ==
-                   cudaSuccess
+    // one spark per block while one block per SM slot (16 of 128 threads) holds them, then up to kSmallSparks
+    const int64_t pairs = (int64_t)count * mtiles, slots = 152 * 16;
+    const int per = (int)(pairs <= slots ? 1 : (pairs / slots < kSmallSparks ? pairs / slots : kSmallSparks));
+    dim3 grid((count + per - 1) / per, mtiles);
+    return launch_pdl(k_fitness_small<8, 16, 3>, grid, dim3(kMT), 0, s, mlp, rows, ld, count, (int32_t)per, idx,
+                      partial) == cudaSuccess
                ? 1
                : -1;
   }

@@ -80,14 +80,20 @@ __device__ __forceinline__ void take_if_before(float& bf, int& bc, float of, int
 // are finite, and whose last improvement I extrapolated over the g_rem =
 // lo_gmax - gen generations left, fmaf(-I, g_rem, f), stays above the run's
 // best-so-far, loses: fitness +infinity, amplitude A0, loser[z] = 1 (its
-// row is re-drawn by k_select_copy).  gens_done is only read here.
+// row is re-drawn by k_select_copy).  gens_done is only read here.  With
+// `partial` (per-sample-tile loss sums [mtiles][count] of the guiding rows)
+// the warp first finishes its firework's guiding fitness as the fitness-
+// finish kernel does and stores it in fit_g (one launch fewer where no elite
+// re-score does it).
 __global__ void __launch_bounds__(kSelThreads) k_select_decide(Problem p, const float* __restrict__ fit_e,
-                                                               const float* __restrict__ fit_g,
+                                                               float* __restrict__ fit_g,
                                                                float* __restrict__ fw_amp, float* __restrict__ fw_f,
                                                                int32_t* __restrict__ winner,
                                                                float* __restrict__ best_f,
                                                                const uint32_t* __restrict__ gens_done,
-                                                               float* __restrict__ f_old, int32_t* __restrict__ loser) {
+                                                               float* __restrict__ f_old, int32_t* __restrict__ loser,
+                                                               const float* __restrict__ partial, int32_t mtiles,
+                                                               int32_t count, float n_f) {
   griddep_wait();
   griddep_launch_dependents();
   const int b = blockIdx.x;
@@ -101,6 +107,13 @@ __global__ void __launch_bounds__(kSelThreads) k_select_decide(Problem p, const 
     const int i = b * p.mu + il;  // global firework
     float bf = 0.0f;
     int bc = -1;
+    if (partial) {
+      for (int q = lane; q < p.m; q += 32) {
+        const int64_t r = (int64_t)i * p.m + q;
+        fit_g[r] = __fdiv_rn(tile_sum(partial, r, count, mtiles), n_f);
+      }
+      __syncwarp();  // the warp reads them back below
+    }
     // the candidates in chunks of kSelChunk per lane, every load of a chunk issued before its compares
     for (int c = lane; c < n_cand; c += 32 * kSelChunk) {
       float v[kSelChunk];
@@ -367,11 +380,13 @@ int launch_rank(const Problem& p, float* fit_e, int32_t* top, int32_t* bottom, c
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 
-int launch_select(const Problem& p, const float* fit_e, const float* fit_g, const float* sparks,
+int launch_select(const Problem& p, const float* fit_e, float* fit_g, const float* sparks,
                   const float* guides, float* fw_x, float* fw_amp, float* fw_f, int32_t* winner, float* best_x,
-                  float* best_f, uint32_t* gens_done, float* f_old, int32_t* loser, cudaStream_t s) {
+                  float* best_f, uint32_t* gens_done, float* f_old, int32_t* loser, cudaStream_t s,
+                  const float* partial, int32_t mtiles, int64_t N) {
   if (launch_pdl(k_select_decide, dim3(p.B), dim3(kSelThreads), 0, s, p, fit_e, fit_g, fw_amp, fw_f, winner, best_f,
-                 (const uint32_t*)gens_done, f_old, loser) != cudaSuccess)
+                 (const uint32_t*)gens_done, f_old, loser, partial, mtiles, (int32_t)((int64_t)p.B * p.mu * p.m),
+                 (float)N) != cudaSuccess)
     return -1;
   if (launch_pdl(k_select_copy, dim3(copy_blocks(p.Dp), p.B * p.mu + p.B), dim3(256), 0, s, p, sparks, guides, fw_x,
                  (const int32_t*)winner, best_x, (const int32_t*)loser, gens_done) != cudaSuccess)

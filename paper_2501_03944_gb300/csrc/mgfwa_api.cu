@@ -94,6 +94,7 @@ struct mgfwa_handle {
   float* gscratch = nullptr;  // backpropagation scratch (GradPlan)
   cudaGraphExec_t refine_exec = nullptr;  // the refinement's kernels, captured once
   bool capturing = false;                 // a graph (its own or a group's) is capturing a generation: no host counters
+  bool grouped_fit = false;               // being captured as a member of a group's grouped fitness launches
   bool grouped = false;                   // member of a group
   int64_t refine_kernels = 0;             // kernels in that graph
   cudaGraphExec_t gen_exec = nullptr;     // one generation (explode .. select), captured at the first step
@@ -253,11 +254,16 @@ bool rescore_on(const mgfwa_t* h) {
 
 // In a captured generation the fitness means are finished by the kernel
 // that first reads them (the explosion sparks' by the rank, the guiding
-// sparks' by the elite pick when the re-score runs), one launch fewer
+// sparks' by the elite pick when the re-score runs, else by the selection), one launch fewer
 // each; phase-by-phase stepping keeps the separate finish so that every
 // phase's buffers can be read.
 bool finish_in_rank(const mgfwa_t* h) { return h->capturing && h->kind == MGFWA_OBJ_MLP_CE; }
 bool finish_in_pick(const mgfwa_t* h) { return h->capturing && rescore_on(h); }
+// (not with lagged guiding, whose one launch's sums are finished before the rank, nor for a member of a grouped
+// fitness launch, whose capture skips the guiding evaluation and finishes its sums itself)
+bool finish_in_select(const mgfwa_t* h) {
+  return h->capturing && !h->grouped_fit && h->kind == MGFWA_OBJ_MLP_CE && !rescore_on(h) && !h->lag_now;
+}
 
 // Generation `gen` (1-based) ends with a hybrid refinement.
 bool refine_due(const mgfwa_t* h, int32_t gen) {
@@ -387,7 +393,7 @@ mgfwa_status run_phase(mgfwa_t* h, int32_t phase) {
     }
     case MGFWA_PHASE_EVAL_G:
       if (h->lag_now) return MGFWA_OK;
-      return eval_rows(h, n_e, p.B * p.mu * p.m, prec, finish_in_pick(h));
+      return eval_rows(h, n_e, p.B * p.mu * p.m, prec, finish_in_pick(h) || finish_in_select(h));
     case MGFWA_PHASE_RESCORE: {
       // low precision: each firework's elite candidates get their fitness in FP32
       const int32_t E = h->cfg.elite_rescore;
@@ -412,7 +418,7 @@ mgfwa_status run_phase(mgfwa_t* h, int32_t phase) {
       Mark mk(h, G_SELECT);
       MG_LAUNCH(h, launch_select(p, h->fit, h->fit + n_e, h->sparks, h->sparks + n_e * p.Dp, h->fw_x, h->fw_amp,
                                  h->fw_f, h->winner, h->best_x, h->best_f, h->gens_done, h->f_old, h->loser,
-                                 h->stream),
+                                 h->stream, finish_in_select(h) ? h->partial : nullptr, h->mtiles, h->mlp.N),
                 "select");
       if (!h->capturing) h->evals += h->P;
       return MGFWA_OK;
@@ -1491,6 +1497,7 @@ mgfwa_status group_capture(mgfwa_group* g, const std::vector<int>& live) {
     cudaStream_t own = h->stream;
     h->stream = br;
     h->capturing = true;
+    h->grouped_fit = is_fused[(size_t)i] != 0;
     const int64_t before = h->launches;
     for (int32_t ph = p0; ph <= p1 && st == MGFWA_OK; ++ph) {
       if (is_fused[(size_t)i] && (ph == MGFWA_PHASE_EVAL_E || ph == MGFWA_PHASE_EVAL_G)) continue;
@@ -1508,6 +1515,7 @@ mgfwa_status group_capture(mgfwa_group* g, const std::vector<int>& live) {
     g->kernels[(size_t)i] += h->launches - before;
     h->launches = before;
     h->capturing = false;
+    h->grouped_fit = false;
     h->stream = own;
     if (st != MGFWA_OK) return false;
     return cudaEventRecord(end, br) == cudaSuccess && cudaStreamWaitEvent(g->stream, end, 0) == cudaSuccess;

@@ -283,10 +283,13 @@ int launch_run_best_init(const Problem& p, const float* fw_x, const float* fw_f,
 // scratch for the fitness before the selection; loser [B*mu]: 1 where a
 // firework lost), then the copies of the winning rows into fw_x and best_x
 // and the losers' new rows; advances gens_done[0] by one (the generation is
-// complete).
-int launch_select(const Problem& p, const float* fit_e, const float* fit_g, const float* sparks,
+// complete).  With `partial` ([mtiles][B*mu*m] per-sample-tile loss sums of
+// the guiding rows, N samples) the selection also finishes the guiding
+// fitness into fit_g first, exactly as launch_fitness_finish would.
+int launch_select(const Problem& p, const float* fit_e, float* fit_g, const float* sparks,
                   const float* guides, float* fw_x, float* fw_amp, float* fw_f, int32_t* winner,
-                  float* best_x, float* best_f, uint32_t* gens_done, float* f_old, int32_t* loser, cudaStream_t s);
+                  float* best_x, float* best_f, uint32_t* gens_done, float* f_old, int32_t* loser, cudaStream_t s,
+                  const float* partial = nullptr, int32_t mtiles = 0, int64_t N = 0);
 
 // FP32 CUDA-core fitness of `count` rows (stride `ld` floats; row r is
 // rows[idx[r]] when idx is given): per-(m-tile, r) partial cross-entropy
