@@ -622,24 +622,36 @@ int launch_l1_fp32x3(const L1Plan& pl, const Mlp& mlp, const int32_t* idx, int32
 // weights W are both given as three BF16 parts, the same six products and
 // three accumulators as above.  One CTA per 128 rows x 128 outputs x one
 // K split of kNetKPer 32-element blocks (splits = ceil(fan_in / 128): a
-// number fixed by the layer's fan-in alone).  With one split the epilogue
-// adds the bias, applies the activation and writes the FP32 output and/or
-// its three BF16 parts (the next tensor-core layer's A); with several, each
-// split's CTA writes its partial sum ((even + odd) + corrections) and a
-// second kernel adds the partials in split order, then the bias.  A row's
-// outputs are sums over its own inputs in an order fixed by the layer's
-// fan-in, so a spark's value does not depend on which rows share the
-// launch.
+// number fixed by the layer's fan-in alone).  Up to kNetCluster splits of a
+// tile form a thread-block cluster: each CTA leaves its partial sum ((even +
+// odd) + corrections) in its shared memory, and after a cluster barrier the
+// CTAs share the tile's columns, each adding the partials of its columns in
+// split order through distributed shared memory, then the bias and the
+// activation, and writing the FP32 output and/or its three BF16 parts (the
+// next tensor-core layer's A).  With more splits the partials go to memory
+// and a second kernel adds them.  A row's outputs are sums over its own
+// inputs in an order fixed by the layer's fan-in, so a spark's value does not
+// depend on which rows share the launch.
+//
+// At 1,040 rows a 512 x 512 layer is 36 tiles x 4 splits: its six products
+// take about 1 us of tensor time, so what bounds it is the latency of one
+// pass -- loads, MMAs, epilogue, the sum -- and the traffic around it.  All
+// of a CTA's K blocks are in flight at once (no ring), the weights' before
+// the previous layer has finished.
 
 namespace {
 
-constexpr int kNetKPer = 4;  // 32-element K blocks per split
+constexpr int kNetKPer = 4;      // 32-element K blocks per split
+constexpr int kNetCluster = 8;   // splits of a tile that meet in one cluster (the portable size)
+constexpr int kNetThreads = 320; // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue (two per TMEM lane quadrant)
+static_assert(kNetKPer <= kStages, "every K block of a split has its own stage");
+static_assert((size_t)kBM * kN * sizeof(float) <= (size_t)kStages * kStageBytes, "partial tile fits in the stages");
 
 struct NetX3Args {
   int32_t rows;        // rows of this launch (A rows [0, rows))
   int32_t k_blocks;    // 32-element K blocks of the fan-in
-  int32_t splits;      // K splits (gridDim.z); > 1: partial sums into `partial`
-  float* partial;      // [splits][rows][n]
+  int32_t splits;      // K splits (gridDim.z)
+  float* partial;      // splits > kNetCluster: partial sums [splits][rows][n]; else null
   int32_t n;           // fan-out
   int32_t act;         // activation, or < 0 for none
   const float* bias;   // [n]
@@ -656,25 +668,79 @@ __device__ __forceinline__ float net_act(int a, float v) {
   return fmaxf(v, 0.0f);
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_to(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+// Outputs col .. col + 7 of row r (z: the sums with the bias not yet added):
+// n is even, so they end at an even count; 16-byte stores where the row
+// starts and n allow.
+__device__ __forceinline__ void net_store8(const NetX3Args& a, int64_t r, int col, const float* z) {
+  float o[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float v = z[i] + (col + i < a.n ? a.bias[col + i] : 0.0f);
+    o[i] = a.act >= 0 ? net_act(a.act, v) : v;
+  }
+  if (a.out) {
+    float* orow = a.out + r * a.ldo + col;
+    if (col + 8 <= a.n && (reinterpret_cast<uintptr_t>(orow) & 15u) == 0) {
+      *reinterpret_cast<float4*>(orow) = make_float4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<float4*>(orow + 4) = make_float4(o[4], o[5], o[6], o[7]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (col + i < a.n) orow[i] = o[i];
+    }
+  }
+  if (a.parts) {
+    uint32_t w[kParts][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) split2(o[2 * i], o[2 * i + 1], w[0][i], w[1][i], w[2][i]);
+    uint32_t* d = a.parts + r * (a.n / 2) + col / 2;
+#pragma unroll
+    for (int p = 0; p < kParts; ++p, d += a.plane_words) {
+      if (col + 8 <= a.n && (reinterpret_cast<uintptr_t>(d) & 15u) == 0) {
+        *reinterpret_cast<uint4*>(d) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (col + 2 * i < a.n) d[i] = w[p][i];
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kNetThreads, 1)
     k_net_x3(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w, NetX3Args a) {
-  griddep_wait();
-  griddep_launch_dependents();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   auto Ap = [&](int p, int s) { return base + ((size_t)s * 2 * kParts + p) * kPartBytes; };
   auto Wp = [&](int p, int s) { return base + ((size_t)s * 2 * kParts + kParts + p) * kPartBytes; };
   Bars* sb = reinterpret_cast<Bars*>(base + (size_t)kStages * kStageBytes);
+  float* part = reinterpret_cast<float*>(base);  // the split's partial tile [column][row], once the MMAs are done
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mt = blockIdx.x, nt = blockIdx.y;
   // this CTA's K blocks [kb0, kb0 + nkb)
   const int kb0 = (int)blockIdx.z * kNetKPer;
   const int nkb = min(kNetKPer, a.k_blocks - kb0);
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&sb->full[s], 1);
-      mbar_init(&sb->empty[s], 1);
-    }
+    for (int s = 0; s < kStages; ++s) mbar_init(&sb->full[s], 1);
     mbar_init(&sb->done, 1);
     sb->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -691,34 +757,33 @@ __global__ void __launch_bounds__(kThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = sb->tmem_base;
 
+  // The weights' parts were written when the handle was made: their copies
+  // start before the previous kernel (the layer's input) has finished.
+  if (warp == 0 && lane == 0) {
+    for (int kb = 0; kb < nkb; ++kb) {
+      mbar_expect_tx(&sb->full[kb], kStageBytes);
+#pragma unroll
+      for (int p = 0; p < kParts; ++p) tma_3d(Wp(p, kb), &tmap_w, (kb0 + kb) * kBKf, nt * kN, p, &sb->full[kb]);
+    }
+  }
+  griddep_wait();
+  griddep_launch_dependents();
   if (warp == 0) {
     if (lane == 0) {
-      int kb = 0;
-      for (; kb < nkb; ++kb) {
-        const int s = kb % kStages;
-        const uint32_t ph = (uint32_t)(kb / kStages) & 1u;
-        if (!mbar_wait(sb, &sb->empty[s], ph ^ 1u, a.status, 1u)) break;
-        mbar_expect_tx(&sb->full[s], kStageBytes);
+      for (int kb = 0; kb < nkb; ++kb)
 #pragma unroll
-        for (int p = 0; p < kParts; ++p) {
-          tma_3d(Ap(p, s), &tmap_a, (kb0 + kb) * kBKf, mt * kBM, p, &sb->full[s]);
-          tma_3d(Wp(p, s), &tmap_w, (kb0 + kb) * kBKf, nt * kN, p, &sb->full[s]);
-        }
-      }
-      for (int j = kb - kStages > 0 ? kb - kStages : 0; j < kb; ++j)
-        mbar_drain(&sb->full[j % kStages], (uint32_t)(j / kStages) & 1u, a.status);
+        for (int p = 0; p < kParts; ++p) tma_3d(Ap(p, kb), &tmap_a, (kb0 + kb) * kBKf, mt * kBM, p, &sb->full[kb]);
+      // every issued copy lands before the CTA may exit
+      for (int kb = 0; kb < nkb; ++kb) mbar_drain(&sb->full[kb], 0u, a.status);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16(kBM, kN);
-      int kb = 0;
-      for (; kb < nkb; ++kb) {
-        const int s = kb % kStages;
-        const uint32_t ph = (uint32_t)(kb / kStages) & 1u;
-        if (!mbar_wait(sb, &sb->full[s], ph, a.status, 2u)) break;
+      for (int kb = 0; kb < nkb; ++kb) {
+        if (!mbar_wait(sb, &sb->full[kb], 0u, a.status, 2u)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t x1 = smem_u32(Ap(0, s)), x2 = smem_u32(Ap(1, s)), x3 = smem_u32(Ap(2, s));
-        const uint32_t w1 = smem_u32(Wp(0, s)), w2 = smem_u32(Wp(1, s)), w3 = smem_u32(Wp(2, s));
+        const uint32_t x1 = smem_u32(Ap(0, kb)), x2 = smem_u32(Ap(1, kb)), x3 = smem_u32(Ap(2, kb));
+        const uint32_t w1 = smem_u32(Wp(0, kb)), w2 = smem_u32(Wp(1, kb)), w3 = smem_u32(Wp(2, kb));
         const uint32_t d_main = tmem + (uint32_t)((kb & 1) * kN), d_corr = tmem + (uint32_t)(2 * kN);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -732,65 +797,70 @@ __global__ void __launch_bounds__(kThreads, 1)
           mma_bf16(d_corr, smem_desc_sw64(x1 + o), smem_desc_sw64(w3 + o), idesc, 1u);
           mma_bf16(d_corr, smem_desc_sw64(x3 + o), smem_desc_sw64(w1 + o), idesc, 1u);
         }
-        mma_commit(&sb->empty[s]);
       }
-      mma_commit(&sb->done);
+      mma_commit(&sb->done);  // after every issued MMA (also on abort)
     }
-  } else {
-    const int q = warp & 3;
-    const int rrow = q * 32 + lane;
+  }
+  const int q = warp & 3, half = (warp - 2) >> 2;  // epilogue warps: TMEM lane quadrant, half of the columns
+  const int rrow = q * 32 + lane;
+  const int64_t r = (int64_t)mt * kBM + rrow;
+  const bool inside = r < a.rows;
+  if (warp >= 2) {
     const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
     mbar_drain(&sb->done, 0u, a.status);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int64_t r = (int64_t)mt * kBM + rrow;
-    const bool valid = !sb->abort_flag && r < a.rows;
     const bool odd = nkb > 1;
-    const int half_n = a.n / 2;
-    const bool split = a.splits > 1;
 #pragma unroll 1
-    for (int j0 = 0; j0 < kN; j0 += 8) {
-      const int col = nt * kN + j0;
-      float x[8], x1[8], xc[8];
-      tmem_ld8(lanes + (uint32_t)j0, x);
-      tmem_ld8(lanes + (uint32_t)(kN + j0), x1);
-      tmem_ld8(lanes + (uint32_t)(2 * kN + j0), xc);
+    for (int j0 = half * (kN / 2); j0 < (half + 1) * (kN / 2); j0 += 16) {
+      float x[16], x1[16], xc[16];
+#pragma unroll
+      for (int h = 0; h < 16; h += 8) {
+        tmem_ld8(lanes + (uint32_t)(j0 + h), x + h);
+        tmem_ld8(lanes + (uint32_t)(kN + j0 + h), x1 + h);
+        tmem_ld8(lanes + (uint32_t)(2 * kN + j0 + h), xc + h);
+      }
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (!valid || col >= a.n) continue;
-      if (split) {
-        // this split's partial sums; the bias and the activation follow the split-ordered sum
-        float* prow = a.partial + ((int64_t)blockIdx.z * a.rows + r) * a.n;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          if (col + i < a.n) prow[col + i] = (odd ? x[i] + x1[i] : x[i]) + xc[i];
-        continue;
-      }
-      float o[8];
+      for (int i = 0; i < 16; ++i) x[i] = (odd ? x[i] + x1[i] : x[i]) + xc[i];
+      if (!a.partial) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float z = ((odd ? x[i] + x1[i] : x[i]) + xc[i]) + (col + i < a.n ? a.bias[col + i] : 0.0f);
-        o[i] = a.act >= 0 ? net_act(a.act, z) : z;
-      }
-      if (a.out) {
-        float* orow = a.out + r * a.ldo;
+        for (int i = 0; i < 16; ++i) part[(j0 + i) * kBM + rrow] = x[i];
+      } else if (inside && !sb->abort_flag) {
+        const int col = nt * kN + j0;
+        float* prow = a.partial + ((int64_t)blockIdx.z * a.rows + r) * a.n + col;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          if (col + i < a.n) orow[col + i] = o[i];
-      }
-      if (a.parts) {
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-          if (col + i >= a.n) break;
-          uint32_t p1, p2, p3;
-          split2(o[i], o[i + 1], p1, p2, p3);
-          uint32_t* d = a.parts + r * half_n + (col + i) / 2;
-          d[0] = p1;
-          d[a.plane_words] = p2;
-          d[2 * a.plane_words] = p3;
-        }
+        for (int i = 0; i < 16; i += 2)
+          if (col + i < a.n) *reinterpret_cast<float2*>(prow + i) = make_float2(x[i], x[i + 1]);
       }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (!a.partial) {
+    __syncwarp();
+    cluster_sync();  // every split's partial tile is in its CTA's shared memory
+    if (warp >= 2) {
+      // this CTA's columns of the tile, eight at a time: the cluster's partials in split order
+      const bool store = inside && !sb->abort_flag;
+      for (int o = (int)cluster_rank() + a.splits * half; o < kN / 8; o += 2 * a.splits) {
+        const int col = nt * kN + o * 8;
+        if (col >= a.n) break;
+        const uint32_t at = smem_u32(part + o * 8 * kBM + rrow);
+        float z[8];
+#pragma unroll 4
+        for (int sp = 0; sp < a.splits; ++sp) {
+          const uint32_t peer = map_to(at, (uint32_t)sp);
+          float v[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = ld_cluster(peer + (uint32_t)(i * kBM * (int)sizeof(float)));
+#pragma unroll
+          for (int i = 0; i < 8; ++i) z[i] = sp == 0 ? v[i] : z[i] + v[i];
+        }
+        if (store) net_store8(a, r, col, z);
+      }
+    }
+    __syncwarp();
+    cluster_sync();  // no CTA leaves while another may still read its tile
+  }
   __syncthreads();
   if (warp == 1) {
     __syncwarp();
@@ -799,8 +869,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// The split layer's outputs: z = ((p_0 + p_1) + ...) + b, activated, into the FP32 output and/or the BF16
-// parts (one thread per pair of outputs of a row).
+// The outputs of a layer with more splits than a cluster holds: z = ((p_0 + p_1) + ...) + b, activated, into the
+// FP32 output and/or the BF16 parts (one thread per pair of outputs of a row).
 __global__ void __launch_bounds__(256) k_net_x3_reduce(NetX3Args a) {
   griddep_wait();
   griddep_launch_dependents();
@@ -836,6 +906,27 @@ __global__ void __launch_bounds__(256) k_net_x3_reduce(NetX3Args a) {
   }
 }
 
+// launch_pdl with clusters of `cz` blocks along z.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_z(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, unsigned cz, cudaStream_t s,
+                         Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 1;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = cz;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 size_t net_x3_smem() { return 1024 + (size_t)kStages * kStageBytes + ((sizeof(Bars) + 15) & ~size_t(15)) + 64; }
 
 }  // namespace
@@ -850,7 +941,7 @@ int64_t net_x3_words(const NetOut& net, int64_t max_rows) {
   for (int l = 0; l < net.n_layers; ++l)
     if (net_x3_layer(net.widths[l], net.widths[l + 1]) && net_x3_splits(net.widths[l]) > ks)
       ks = net_x3_splits(net.widths[l]);
-  if (ks > 1) w += (int64_t)ks * max_rows * net.wmax;  // the split layers' FP32 partial sums
+  if (ks > kNetCluster) w += (int64_t)ks * max_rows * net.wmax;  // FP32 partial sums
   for (int l = 0; l < net.n_layers; ++l)
     if (net_x3_layer(net.widths[l], net.widths[l + 1])) w += 3 * (int64_t)net.widths[l + 1] * (net.widths[l] / 2);
   return w;
@@ -874,7 +965,7 @@ bool net_x3_plan(NetX3Plan& pl, const NetOut& net, int64_t max_rows, uint32_t* b
   for (int l = 0; l < net.n_layers; ++l)
     if (net_x3_layer(net.widths[l], net.widths[l + 1]) && net_x3_splits(net.widths[l]) > ks)
       ks = net_x3_splits(net.widths[l]);
-  if (ks > 1) {
+  if (ks > kNetCluster) {
     pl.partial = reinterpret_cast<float*>(wcur);
     wcur += (int64_t)ks * max_rows * net.wmax;
   }
@@ -951,7 +1042,7 @@ int launch_net_output_x3(const NetX3Plan& pl, const NetOut& net, const float* ro
       x.rows = count;
       x.k_blocks = (fi + kBKf - 1) / kBKf;
       x.splits = net_x3_splits(fi);
-      x.partial = pl.partial;
+      x.partial = x.splits > kNetCluster ? pl.partial : nullptr;
       x.n = fo;
       x.act = ak;
       x.bias = b;
@@ -961,11 +1052,11 @@ int launch_net_output_x3(const NetX3Plan& pl, const NetOut& net, const float* ro
       x.plane_words = pl.max_rows * (fo / 2);
       x.status = status;
       const dim3 grid((unsigned)((count + kBM - 1) / kBM), (unsigned)((fo + kN - 1) / kN), (unsigned)x.splits);
-      if (launch_pdl(k_net_x3, grid, dim3(kThreads), net_x3_smem(), s, pl.tmap_a[l], pl.tmap_w[l], x) !=
-          cudaSuccess)
+      if (launch_pdl_z(k_net_x3, grid, dim3(kNetThreads), net_x3_smem(), x.partial ? 1u : (unsigned)x.splits, s,
+                       pl.tmap_a[l], pl.tmap_w[l], x) != cudaSuccess)
         return -1;
       ++n;
-      if (x.splits > 1) {
+      if (x.partial) {
         const int64_t pairs = (int64_t)count * (fo / 2);
         const unsigned blocks = (unsigned)((pairs + 255) / 256 < 4096 ? (pairs + 255) / 256 : 4096);
         if (launch_pdl(k_net_x3_reduce, dim3(blocks), dim3(256), 0, s, x) != cudaSuccess) return -1;
