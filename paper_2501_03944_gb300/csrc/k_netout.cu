@@ -17,17 +17,18 @@ namespace mgfwa {
 namespace {
 
 constexpr int kBK = 16;      // k-slab depth
-constexpr int kStages = 3;   // slabs in flight per group (cp.async ring)
 constexpr int kTN = 32;      // output tile columns per block
 constexpr int kGroups = 4;   // fan-in chunks, one per 64-thread group
-constexpr int kPadW = kTN + 4;
+constexpr int kPadK = kBK + 4;   // slab row stride: eight rows' float4s lie in distinct banks
+constexpr int kPadW = kTN + 8;   // partial tile row stride
 
-// Tile geometry for TR output rows per thread: 8 TR rows x 32 columns per block.
-template <int TR>
+// Tile geometry for TR output rows per thread: 8 TR rows x 32 columns per
+// block, ST slabs of A and W in flight per group (cp.async ring).
+template <int TR, int ST>
 struct NetTile {
   static constexpr int kTM = 8 * TR;
-  static constexpr int kPadA = kTM + 4;
-  static constexpr int kGroupFloats = kStages * kBK * (kPadA + kPadW);  // the ring of A and W slabs per group
+  static constexpr int kSlab = (kTM + kTN) * kPadK;  // A rows, then W rows, k contiguous
+  static constexpr int kGroupFloats = ST * kSlab;
   static constexpr size_t kSmem = sizeof(float) * kGroups * kGroupFloats;
   static_assert(kTM * kPadW <= kGroupFloats, "partial tiles must fit in the slab space");
 };
@@ -38,11 +39,15 @@ __device__ __forceinline__ float act32(int a, float v) {
   return fmaxf(v, 0.0f);
 }
 
-// 4-byte asynchronous global -> shared copy; src_bytes = 0 writes a zero
-// without reading (the source address must still be a valid one).
+// 4- and 16-byte asynchronous global -> shared copies; src_bytes = 0 writes
+// zeros without reading (the source address must still be a valid one).
 __device__ __forceinline__ void cp_async4(float* dst, const float* src, uint32_t src_bytes) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, uint32_t src_bytes) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -54,27 +59,27 @@ __host__ __device__ __forceinline__ int chunk_len(int k) { return kBK * ((k + kB
 // out[r][j] = act(sum_i A[r][i] W[j][i] + b[j]) (no activation when act < 0)
 // for r < rows, j < n; A row stride lda, out row stride ldo.  One 256-thread
 // block per (8 TR) x 32 output tile.  Group g (threads 64 g ..) multiplies
-// the tile over its fan-in chunk, TR x 4 outputs per thread:
-// k-slabs of A and W are copied asynchronously (4-byte cp.async, transposed
-// to k-major so a thread's rows and columns are contiguous) into the group's
-// ring of kStages slabs, two slabs in flight while one is multiplied, one
-// group barrier per slab.  The four partial tiles then meet in shared memory
-// and every thread adds them in group order for TR of the tile's outputs,
-// adds the bias and applies the activation.  A quarter of the fan-in per group cuts each
-// block's serial slab chain to a quarter, which is what bounds the small-row
-// launches (the guiding sparks).  TR = 8 takes three 16-byte shared loads per
-// 32 FMAs (for launches that fill the SMs), TR = 4 two per 16 with twice the
-// blocks.  Both compute every output with the same operations in the same
-// order, so the choice never changes a result.
-template <int TR>
-__global__ void __launch_bounds__(256, TR == 4 ? 4 : 2) k_net_layer(const float* __restrict__ A, int64_t lda, int32_t rows,
-                                                   const float* __restrict__ W, const float* __restrict__ bias,
-                                                   int32_t k, int32_t n, int32_t act, float* __restrict__ out,
-                                                   int64_t ldo) {
-  constexpr int kTM = NetTile<TR>::kTM, kPadA = NetTile<TR>::kPadA, kGroupFloats = NetTile<TR>::kGroupFloats;
-  griddep_wait();
-  griddep_launch_dependents();
-  // slabs [group][stage]{A [kBK][kPadA], W [kBK][kPadW]}; afterwards the partial tiles [group][kTM][kPadW]
+// the tile over its fan-in chunk, TR x 4 outputs per thread (rows ty + 8 i,
+// columns tx + 8 j): k-slabs of A and W rows are copied asynchronously into
+// the group's ring of ST slabs as they lie in memory (V4: 16 bytes at a
+// time, else 4), ST - 1 slabs in flight while one is multiplied, one group
+// barrier per slab; a thread reads four k of a row per 16-byte shared load.
+// The four partial tiles then meet in shared memory and every thread adds
+// them in group order for TR of the tile's outputs, adds the bias and applies
+// the activation.  A quarter of the fan-in per group cuts each block's serial
+// slab chain to a quarter, which is what bounds the small-row launches (the
+// guiding sparks).  The weights do not depend on the previous kernel, so the
+// first slabs' W rows are copied before its end is waited for.  Every shape
+// computes every output with the same operations in the same order, so the
+// choice never changes a result.
+template <int TR, int ST, bool V4>
+__global__ void __launch_bounds__(256, TR == 8 ? 2 : TR == 4 ? 3 : 2)
+    k_net_layer(const float* __restrict__ A, int64_t lda, int32_t rows, const float* __restrict__ W,
+                const float* __restrict__ bias, int32_t k, int32_t n, int32_t act, float* __restrict__ out,
+                int64_t ldo) {
+  using Tile = NetTile<TR, ST>;
+  constexpr int kTM = Tile::kTM, kW = V4 ? 4 : 1;  // floats per copy
+  // slabs [group][stage]{A [kTM][kPadK], W [kTN][kPadK]}; afterwards the partial tiles [group][kTM][kPadW]
   extern __shared__ __align__(16) float sm[];
   const int g = threadIdx.x >> 6, t = threadIdx.x & 63;
   const int tx = t & 7, ty = t >> 3;
@@ -82,36 +87,30 @@ __global__ void __launch_bounds__(256, TR == 4 ? 4 : 2) k_net_layer(const float*
   const int c = chunk_len(k);
   const int kbeg = g * c, kend = min(kbeg + c, k);
   const int slabs = kend > kbeg ? (kend - kbeg + kBK - 1) / kBK : 0;
-  float* const base = sm + g * kGroupFloats;
-  auto As = [&](int stage) { return base + stage * kBK * (kPadA + kPadW); };
-  auto Ws = [&](int stage) { return base + stage * kBK * (kPadA + kPadW) + kBK * kPadA; };
-  constexpr int LA = kTM * kBK / 64, LW = kTN * kBK / 64;  // slab elements each thread copies
-  // element q of a thread is (row rq + 4 q, column kq) of the slab: 16
-  // neighbouring threads read 16 consecutive floats of one row
-  const int kq = t % kBK, rq = t / kBK;
-  const float* pa = A + (int64_t)(r0 + rq) * lda + kq;  // dereferenced only where in range
-  const float* pw = W + (int64_t)(j0 + rq) * k + kq;
-  const int64_t sa = 4 * lda, sw = 4 * (int64_t)k;
-  unsigned va = 0, vw = 0;
+  float* const base = sm + g * Tile::kGroupFloats;
+  // a thread copies k offset kq of slab rows rq, rq + kRows, ...: neighbouring
+  // threads read one row's consecutive floats
+  constexpr int kPer = kBK / kW, kRows = 64 / kPer;
+  const int kq = (t % kPer) * kW, rq = t / kPer;
+  auto copy = [&](float* dst, const float* src, bool in, const float* safe) {
+    if (V4)
+      cp_async16(dst, in ? src : safe, in ? 16u : 0u);
+    else
+      cp_async4(dst, in ? src : safe, in ? 4u : 0u);
+  };
+  auto fetch_w = [&](int slab, int stage) {
+    const int k0 = kbeg + slab * kBK + kq;
+    float* w = base + stage * Tile::kSlab + kTM * kPadK + kq;
 #pragma unroll
-  for (int q = 0; q < LA; ++q) va |= (r0 + rq + 4 * q < rows ? 1u : 0u) << q;
+    for (int q = rq; q < kTN; q += kRows)
+      copy(w + q * kPadK, W + (int64_t)(j0 + q) * k + k0, k0 < kend && j0 + q < n, W);
+  };
+  auto fetch_a = [&](int slab, int stage) {
+    const int k0 = kbeg + slab * kBK + kq;
+    float* a = base + stage * Tile::kSlab + kq;
 #pragma unroll
-  for (int q = 0; q < LW; ++q) vw |= (j0 + rq + 4 * q < n ? 1u : 0u) << q;
-  auto fetch = [&](int slab, int stage) {
-    const int k0 = kbeg + slab * kBK;
-    const bool kin = k0 + kq < kend;
-    float* a = As(stage) + kq * kPadA + rq;
-    float* w = Ws(stage) + kq * kPadW + rq;
-#pragma unroll
-    for (int q = 0; q < LA; ++q) {
-      const bool in = kin && (va >> q & 1u);
-      cp_async4(a + 4 * q, in ? pa + q * sa + k0 : A, in ? 4u : 0u);
-    }
-#pragma unroll
-    for (int q = 0; q < LW; ++q) {
-      const bool in = kin && (vw >> q & 1u);
-      cp_async4(w + 4 * q, in ? pw + q * sw + k0 : W, in ? 4u : 0u);
-    }
+    for (int q = rq; q < kTM; q += kRows)
+      copy(a + q * kPadK, A + (int64_t)(r0 + q) * lda + k0, k0 < kend && r0 + q < rows, A);
   };
   auto group_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(g + 1) : "memory"); };
   float acc[TR][4];
@@ -120,34 +119,40 @@ __global__ void __launch_bounds__(256, TR == 4 ? 4 : 2) k_net_layer(const float*
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
 #pragma unroll
-  for (int i = 0; i < kStages - 1; ++i) {
-    if (i < slabs) fetch(i, i);
-    cp_async_commit();
+  for (int i = 0; i < ST - 1; ++i)
+    if (i < slabs) fetch_w(i, i);
+  griddep_wait();
+  griddep_launch_dependents();
+#pragma unroll
+  for (int i = 0; i < ST - 1; ++i) {
+    if (i < slabs) fetch_a(i, i);
+    cp_async_commit();  // the first of these groups also holds the W copies above
   }
   for (int s = 0; s < slabs; ++s) {
-    const int cur = s % kStages;
-    cp_async_wait<kStages - 2>();  // this thread's copies of slab s have landed
-    group_sync();                  // everyone's have; everyone is done with slab s - 1
-    const float* a = As(cur);
-    const float* w = Ws(cur);
+    cp_async_wait<ST - 2>();  // this thread's copies of slab s have landed
+    group_sync();             // everyone's have; everyone is done with slab s - 1
+    const float* a = base + (s % ST) * Tile::kSlab + ty * kPadK;
+    const float* w = base + (s % ST) * Tile::kSlab + (kTM + tx) * kPadK;
 #pragma unroll
-    for (int kk = 0; kk < kBK; ++kk) {
-      float ai[TR];
+    for (int kk = 0; kk < kBK; kk += 4) {
+      float4 av[TR], wv[4];
 #pragma unroll
-      for (int h = 0; h < TR / 4; ++h) {
-        const float4 av = *reinterpret_cast<const float4*>(a + kk * kPadA + ty * TR + 4 * h);
-        ai[4 * h] = av.x; ai[4 * h + 1] = av.y; ai[4 * h + 2] = av.z; ai[4 * h + 3] = av.w;
-      }
-      const float4 wv = *reinterpret_cast<const float4*>(w + kk * kPadW + tx * 4);
-      const float wj[4] = {wv.x, wv.y, wv.z, wv.w};
+      for (int i = 0; i < TR; ++i) av[i] = *reinterpret_cast<const float4*>(a + 8 * i * kPadK + kk);
 #pragma unroll
-      for (int i = 0; i < TR; ++i)
+      for (int j = 0; j < 4; ++j) wv[j] = *reinterpret_cast<const float4*>(w + 8 * j * kPadK + kk);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ai[i], wj[j], acc[i][j]);
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(lane_of(av[i], u), lane_of(wv[j], u), acc[i][j]);
     }
-    // the ring slot of slab s + kStages - 1 last held slab s - 1, which every
+    // the ring slot of slab s + ST - 1 last held slab s - 1, which every
     // thread of the group finished before the barrier above
-    if (s + kStages - 1 < slabs) fetch(s + kStages - 1, (s + kStages - 1) % kStages);
+    if (s + ST - 1 < slabs) {
+      fetch_w(s + ST - 1, (s + ST - 1) % ST);
+      fetch_a(s + ST - 1, (s + ST - 1) % ST);
+    }
     cp_async_commit();
   }
   cp_async_wait<0>();
@@ -155,8 +160,8 @@ __global__ void __launch_bounds__(256, TR == 4 ? 4 : 2) k_net_layer(const float*
   float* part = sm + g * (kTM * kPadW);
 #pragma unroll
   for (int i = 0; i < TR; ++i)
-    *reinterpret_cast<float4*>(part + (ty * TR + i) * kPadW + tx * 4) =
-        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) part[(ty + 8 * i) * kPadW + tx + 8 * j] = acc[i][j];
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < kTM * kTN / 256; ++q) {
@@ -206,24 +211,41 @@ __global__ void __launch_bounds__(32 * kF64Warps) k_net_f64_layer(const float* _
 
 }  // namespace
 
+namespace {
+template <int TR, int ST, bool V4>
+cudaError_t net_layer(const float* a, int64_t lda, int32_t count, const float* W, const float* b, int32_t fi,
+                      int32_t fo, int32_t ak, float* o, int64_t ldo, cudaStream_t s) {
+  using Tile = NetTile<TR, ST>;
+  const cudaError_t e = ensure_smem_limit<k_net_layer<TR, ST, V4>>(Tile::kSmem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_net_layer<TR, ST, V4>,
+                    dim3((unsigned)((count + Tile::kTM - 1) / Tile::kTM), (unsigned)((fo + kTN - 1) / kTN)), dim3(256),
+                    Tile::kSmem, s, a, lda, count, W, b, fi, fo, ak, o, ldo);
+}
+}  // namespace
+
 int launch_net_layer(const float* a, int64_t lda, int32_t count, const float* W, const float* b, int32_t fi,
                      int32_t fo, int32_t ak, float* o, int64_t ldo, cudaStream_t s) {
-  if (ensure_smem_limit<k_net_layer<8>>(NetTile<8>::kSmem) != cudaSuccess ||
-      ensure_smem_limit<k_net_layer<4>>(NetTile<4>::kSmem) != cudaSuccess)
-    return -1;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
                                                  cudaSuccess)
     return -1;
-  // 64-row tiles where they fill the SMs, else 32-row tiles (twice the blocks)
-  const bool wide = (int64_t)((count + 63) / 64) * ((fo + kTN - 1) / kTN) >= sms;
+  // 16-byte copies where every row of both operands starts on 16 bytes (a
+  // chunk starts at a multiple of 16, and k % 4 == 0 makes its end whole)
+  const bool v4 = fi % 4 == 0 && lda % 4 == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(W)) & 15u) == 0;
+  // 64-row tiles where they fill the SMs, else 32-row tiles where those do,
+  // else 8-row tiles with eight slabs in flight (few rows: latency-bound)
+  const int64_t cols = (fo + kTN - 1) / kTN;
   cudaError_t e;
-  if (wide)
-    e = launch_pdl(k_net_layer<8>, dim3((unsigned)((count + 63) / 64), (unsigned)((fo + kTN - 1) / kTN)), dim3(256),
-                   NetTile<8>::kSmem, s, a, lda, count, W, b, fi, fo, ak, o, ldo);
+  if ((int64_t)((count + 63) / 64) * cols >= sms)
+    e = v4 ? net_layer<8, 3, true>(a, lda, count, W, b, fi, fo, ak, o, ldo, s)
+           : net_layer<8, 3, false>(a, lda, count, W, b, fi, fo, ak, o, ldo, s);
+  else if ((int64_t)((count + 31) / 32) * cols >= sms)
+    e = v4 ? net_layer<4, 3, true>(a, lda, count, W, b, fi, fo, ak, o, ldo, s)
+           : net_layer<4, 3, false>(a, lda, count, W, b, fi, fo, ak, o, ldo, s);
   else
-    e = launch_pdl(k_net_layer<4>, dim3((unsigned)((count + 31) / 32), (unsigned)((fo + kTN - 1) / kTN)), dim3(256),
-                   NetTile<4>::kSmem, s, a, lda, count, W, b, fi, fo, ak, o, ldo);
+    e = v4 ? net_layer<1, 8, true>(a, lda, count, W, b, fi, fo, ak, o, ldo, s)
+           : net_layer<1, 8, false>(a, lda, count, W, b, fi, fo, ak, o, ldo, s);
   return e == cudaSuccess ? 1 : -1;
 }
 
