@@ -239,7 +239,7 @@ mgfwa_status eval_rows(mgfwa_t* h, int64_t first, int32_t count, int32_t precisi
                                      h->status, h->stream),
                 "tensor-core fitness");
     else
-      MG_LAUNCH(h, launch_fitness_simt_main(h->mlp, rows, h->p.Dp, count, h->partial, h->stream), "FP32 fitness");
+      MG_LAUNCH(h, launch_fitness_fp32(h->mlp, rows, h->p.Dp, count, h->partial, h->status, h->stream), "FP32 fitness");
   }
   if (defer_finish) return MGFWA_OK;
   Mark mk(h, G_FINISH);
