@@ -270,67 +270,112 @@ __global__ void __launch_bounds__(256) k_sphere(const float* __restrict__ rows, 
   }
 }
 
-// FP64 forward of kF64Samples samples per block (so that every weight read
-// feeds that many FMAs); one warp per output unit, lanes striding over the
-// inputs in index order, then a fixed xor tree per sample.
-constexpr int kF64Samples = 4;
+// FP64 forward of ns (<= kF64Samples) samples per block.  The FP64 pipe is
+// what bounds it (about two FMAs a clock per SM, conversions from FP32 on the
+// same pipe), so it should carry little else: 64 units x 32 inputs of a layer's
+// weights (and, in the first layer, the samples' inputs) are converted once
+// into shared memory, the next slab's loads in flight meanwhile, and each
+// thread sums up to four (unit, sample) outputs, no lane reductions.  Each
+// slab of 32 inputs is a chain of its own from zero in index order and the
+// slabs are added in order, so the rounding error grows like a tree's.  The
+// launcher picks ns so that the blocks fill whole waves of the SMs.  A run's
+// read-back of the 784-64-10 network (N = 2048) 431 -> 306 us with it, of
+// 3072-128-64-10 (N = 4096) 4,366 -> 3,290 us; before, four samples a block,
+// a fifth of the pipe went to lane reductions and a quarter to conversions.
+constexpr int kF64Samples = 16;
+constexpr int kF64Units = 64, kF64K = 32, kF64Threads = 256;
+constexpr int kF64Out = kF64Samples * kF64Units / kF64Threads;  // outputs per thread
 
-__global__ void __launch_bounds__(256) k_fitness_f64(Mlp mlp, const float* __restrict__ x, int wmax,
-                                                     double* __restrict__ ce64) {
+__global__ void __launch_bounds__(kF64Threads) k_fitness_f64(Mlp mlp, const float* __restrict__ x, int ns, int wmax,
+                                                             double* __restrict__ ce64) {
   griddep_wait();
   griddep_launch_dependents();
   extern __shared__ double sd[];
-  double* a = sd;                          // [kF64Samples][wmax]
-  double* b = sd + (size_t)kF64Samples * wmax;
-  const int64_t n0 = (int64_t)blockIdx.x * kF64Samples;
-  const int ns = (int)(mlp.N - n0 < kF64Samples ? mlp.N - n0 : kF64Samples);
-  const int d_in = mlp.widths[0];
-  for (int e = threadIdx.x; e < kF64Samples * d_in; e += blockDim.x) {
-    const int q = e / d_in, i = e - q * d_in;
-    a[q * wmax + i] = q < ns ? (double)mlp.X[(n0 + q) * d_in + i] : 0.0;
-  }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  double* ws = sd;                                  // [kF64Units][kF64K + 1]
+  double* xs = ws + kF64Units * (kF64K + 1);        // [kF64K][kF64Samples]
+  double* a = xs + kF64K * kF64Samples;             // [wmax][kF64Samples], wmax the widest layer output
+  double* b = a + (size_t)wmax * kF64Samples;
+  const int tid = threadIdx.x;
+  const int64_t n0 = (int64_t)blockIdx.x * ns;
   const int L = mlp.n_layers;
+  constexpr int kWL = kF64Units * kF64K / kF64Threads, kXL = kF64Samples * kF64K / kF64Threads;
   for (int l = 0; l < L; ++l) {
     const int fi = mlp.widths[l], fo = mlp.widths[l + 1];
-    const float* W = x + mlp.w_off[l];
-    const float* bias = x + mlp.b_off[l];
-    for (int j = warp; j < fo; j += nwarps) {
-      double s[kF64Samples];
+    for (int u0 = 0; u0 < fo; u0 += kF64Units) {
+      const int uc = min(kF64Units, fo - u0);
+      const float* W = x + mlp.w_off[l] + (int64_t)u0 * fi;
+      float wr[kWL], xr[kXL];
+      auto fetch = [&](int k0) {
 #pragma unroll
-      for (int q = 0; q < kF64Samples; ++q) s[q] = 0.0;
-      for (int i = lane; i < fi; i += 32) {
-        const double wv = (double)W[(int64_t)j * fi + i];
+        for (int i = 0; i < kWL; ++i) {
+          const int e = tid + kF64Threads * i, u = e / kF64K, k = k0 + e % kF64K;
+          wr[i] = u < uc && k < fi ? W[(int64_t)u * fi + k] : 0.0f;
+        }
+        if (l == 0) {
 #pragma unroll
-        for (int q = 0; q < kF64Samples; ++q) s[q] += wv * a[q * wmax + i];
+          for (int i = 0; i < kXL; ++i) {
+            const int e = tid + kF64Threads * i, q = e / kF64K, k = k0 + e % kF64K;
+            xr[i] = q < ns && n0 + q < mlp.N && k < fi ? mlp.X[(n0 + q) * fi + k] : 0.0f;
+          }
+        }
+      };
+      int unit[kF64Out], smp[kF64Out];
+      double acc[kF64Out];
+#pragma unroll
+      for (int q = 0; q < kF64Out; ++q) {
+        const int o = tid + kF64Threads * q;
+        unit[q] = o / ns;
+        smp[q] = o - unit[q] * ns;
+        acc[q] = 0.0;
+      }
+      fetch(0);
+      for (int k0 = 0; k0 < fi; k0 += kF64K) {
+        __syncthreads();  // the slab before has been read
+#pragma unroll
+        for (int i = 0; i < kWL; ++i) {
+          const int e = tid + kF64Threads * i;
+          ws[e / kF64K * (kF64K + 1) + e % kF64K] = (double)wr[i];
+        }
+        if (l == 0) {
+#pragma unroll
+          for (int i = 0; i < kXL; ++i) {
+            const int e = tid + kF64Threads * i;
+            xs[e % kF64K * kF64Samples + e / kF64K] = (double)xr[i];
+          }
+        }
+        __syncthreads();
+        if (k0 + kF64K < fi) fetch(k0 + kF64K);
+        const int kk = min(kF64K, fi - k0);
+        const double* in = l == 0 ? xs : a + (size_t)k0 * kF64Samples;
+#pragma unroll
+        for (int q = 0; q < kF64Out; ++q) {
+          if (unit[q] >= uc) continue;
+          const double* wq = ws + unit[q] * (kF64K + 1);
+          double p = 0.0;
+#pragma unroll 8
+          for (int k = 0; k < kk; ++k) p += wq[k] * in[k * kF64Samples + smp[q]];
+          acc[q] += p;
+        }
       }
 #pragma unroll
-      for (int q = 0; q < kF64Samples; ++q) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], off);
-      }
-      if (lane < kF64Samples) {
-        double v = s[0];
-#pragma unroll
-        for (int q = 1; q < kF64Samples; ++q) v = lane == q ? s[q] : v;
-        v += (double)bias[j];
+      for (int q = 0; q < kF64Out; ++q) {
+        if (unit[q] >= uc) continue;
+        double v = acc[q] + (double)x[mlp.b_off[l] + u0 + unit[q]];
         if (l + 1 < L) v = mlp.acts[l] == kActTanh ? tanh(v) : (v > 0.0 ? v : 0.0);
-        b[lane * wmax + j] = v;
+        b[(u0 + unit[q]) * kF64Samples + smp[q]] = v;
       }
     }
     __syncthreads();
     double* t = a; a = b; b = t;
   }
-  if (threadIdx.x < ns) {
-    const int q = threadIdx.x;
-    const double* z = a + q * wmax;
+  if (tid < ns && n0 + tid < mlp.N) {
+    const double* z = a + tid;
     const int C = mlp.widths[L];
     double zmax = z[0];
-    for (int c = 1; c < C; ++c) zmax = z[c] > zmax ? z[c] : zmax;
+    for (int c = 1; c < C; ++c) zmax = z[c * kF64Samples] > zmax ? z[c * kF64Samples] : zmax;
     double se = 0.0;
-    for (int c = 0; c < C; ++c) se += exp(z[c] - zmax);
-    ce64[n0 + q] = (zmax + log(se)) - z[mlp.y[n0 + q]];
+    for (int c = 0; c < C; ++c) se += exp(z[c * kF64Samples] - zmax);
+    ce64[n0 + tid] = (zmax + log(se)) - z[mlp.y[n0 + tid] * kF64Samples];
   }
 }
 
@@ -406,11 +451,17 @@ int launch_fitness_sphere(const float* rows, int64_t ld, int64_t D, int32_t coun
 }
 
 int launch_fitness_f64(const Mlp& mlp, const float* x, double* ce64, double* out, cudaStream_t s) {
-  int wmax = 0;
-  for (int l = 0; l <= mlp.n_layers; ++l) wmax = wmax > mlp.widths[l] ? wmax : mlp.widths[l];
-  const size_t smem = 2 * sizeof(double) * (size_t)kF64Samples * wmax;
+  int dev = 0, sms = 0, wmax = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return -1;
+  for (int l = 1; l <= mlp.n_layers; ++l) wmax = wmax > mlp.widths[l] ? wmax : mlp.widths[l];
+  const int64_t waves = (mlp.N + (int64_t)kF64Samples * sms - 1) / ((int64_t)kF64Samples * sms);
+  const int ns = (int)((mlp.N + waves * sms - 1) / (waves * sms));
+  const size_t smem = sizeof(double) * ((size_t)kF64Units * (kF64K + 1) + (size_t)kF64K * kF64Samples +
+                                        2 * (size_t)wmax * kF64Samples);
   if (smem > 48 * 1024 && ensure_smem_limit<k_fitness_f64>(smem) != cudaSuccess) return -1;
-  k_fitness_f64<<<(unsigned)((mlp.N + kF64Samples - 1) / kF64Samples), 256, smem, s>>>(mlp, x, wmax, ce64);
+  k_fitness_f64<<<(unsigned)((mlp.N + ns - 1) / ns), kF64Threads, smem, s>>>(mlp, x, ns, wmax, ce64);
   if (cudaPeekAtLastError() != cudaSuccess) return -1;
   k_reduce_f64<<<1, 256, 0, s>>>(ce64, nullptr, mlp.N, 1.0 / (double)mlp.N, out);
   return cudaPeekAtLastError() == cudaSuccess ? 2 : -1;
