@@ -17,16 +17,15 @@ namespace mgfwa {
 namespace {
 
 constexpr int kBK = 16;      // k-slab depth
-constexpr int kTN = 32;      // output tile columns per block
 constexpr int kGroups = 4;   // fan-in chunks, one per 64-thread group
 constexpr int kPadK = kBK + 4;   // slab row stride: eight rows' float4s lie in distinct banks
-constexpr int kPadW = kTN + 8;   // partial tile row stride
 
-// Tile geometry for TR output rows per thread: 8 TR rows x 32 columns per
+// Tile geometry for TR x TC outputs per thread: 8 TR rows x 8 TC columns per
 // block, ST slabs of A and W in flight per group (cp.async ring).
-template <int TR, int ST>
+template <int TR, int TC, int ST>
 struct NetTile {
-  static constexpr int kTM = 8 * TR;
+  static constexpr int kTM = 8 * TR, kTN = 8 * TC;
+  static constexpr int kPadW = kTN + 8;                // partial tile row stride
   static constexpr int kSlab = (kTM + kTN) * kPadK;  // A rows, then W rows, k contiguous
   static constexpr int kGroupFloats = ST * kSlab;
   static constexpr size_t kSmem = sizeof(float) * kGroups * kGroupFloats;
@@ -58,8 +57,8 @@ __host__ __device__ __forceinline__ int chunk_len(int k) { return kBK * ((k + kB
 
 // out[r][j] = act(sum_i A[r][i] W[j][i] + b[j]) (no activation when act < 0)
 // for r < rows, j < n; A row stride lda, out row stride ldo.  One 256-thread
-// block per (8 TR) x 32 output tile.  Group g (threads 64 g ..) multiplies
-// the tile over its fan-in chunk, TR x 4 outputs per thread (rows ty + 8 i,
+// block per (8 TR) x (8 TC) output tile.  Group g (threads 64 g ..) multiplies
+// the tile over its fan-in chunk, TR x TC outputs per thread (rows ty + 8 i,
 // columns tx + 8 j): k-slabs of A and W rows are copied asynchronously into
 // the group's ring of ST slabs as they lie in memory (V4: 16 bytes at a
 // time, else 4), ST - 1 slabs in flight while one is multiplied, one group
@@ -72,13 +71,13 @@ __host__ __device__ __forceinline__ int chunk_len(int k) { return kBK * ((k + kB
 // first slabs' W rows are copied before its end is waited for.  Every shape
 // computes every output with the same operations in the same order, so the
 // choice never changes a result.
-template <int TR, int ST, bool V4>
-__global__ void __launch_bounds__(256, TR == 8 ? 2 : TR == 4 ? 3 : 2)
+template <int TR, int TC, int ST, bool V4>
+__global__ void __launch_bounds__(256, TR * TC > 32 ? 1 : TR == 4 ? 3 : 2)
     k_net_layer(const float* __restrict__ A, int64_t lda, int32_t rows, const float* __restrict__ W,
                 const float* __restrict__ bias, int32_t k, int32_t n, int32_t act, float* __restrict__ out,
                 int64_t ldo) {
-  using Tile = NetTile<TR, ST>;
-  constexpr int kTM = Tile::kTM, kW = V4 ? 4 : 1;  // floats per copy
+  using Tile = NetTile<TR, TC, ST>;
+  constexpr int kTM = Tile::kTM, kTN = Tile::kTN, kPadW = Tile::kPadW, kW = V4 ? 4 : 1;  // kW floats per copy
   // slabs [group][stage]{A [kTM][kPadK], W [kTN][kPadK]}; afterwards the partial tiles [group][kTM][kPadW]
   extern __shared__ __align__(16) float sm[];
   const int g = threadIdx.x >> 6, t = threadIdx.x & 63;
@@ -113,11 +112,11 @@ __global__ void __launch_bounds__(256, TR == 8 ? 2 : TR == 4 ? 3 : 2)
       copy(a + q * kPadK, A + (int64_t)(r0 + q) * lda + k0, k0 < kend && r0 + q < rows, A);
   };
   auto group_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(g + 1) : "memory"); };
-  float acc[TR][4];
+  float acc[TR][TC];
 #pragma unroll
   for (int i = 0; i < TR; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+    for (int j = 0; j < TC; ++j) acc[i][j] = 0.0f;
 #pragma unroll
   for (int i = 0; i < ST - 1; ++i)
     if (i < slabs) fetch_w(i, i);
@@ -135,17 +134,17 @@ __global__ void __launch_bounds__(256, TR == 8 ? 2 : TR == 4 ? 3 : 2)
     const float* w = base + (s % ST) * Tile::kSlab + (kTM + tx) * kPadK;
 #pragma unroll
     for (int kk = 0; kk < kBK; kk += 4) {
-      float4 av[TR], wv[4];
+      float4 av[TR], wv[TC];
 #pragma unroll
       for (int i = 0; i < TR; ++i) av[i] = *reinterpret_cast<const float4*>(a + 8 * i * kPadK + kk);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) wv[j] = *reinterpret_cast<const float4*>(w + 8 * j * kPadK + kk);
+      for (int j = 0; j < TC; ++j) wv[j] = *reinterpret_cast<const float4*>(w + 8 * j * kPadK + kk);
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int i = 0; i < TR; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(lane_of(av[i], u), lane_of(wv[j], u), acc[i][j]);
+          for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(lane_of(av[i], u), lane_of(wv[j], u), acc[i][j]);
     }
     // the ring slot of slab s + ST - 1 last held slab s - 1, which every
     // thread of the group finished before the barrier above
@@ -161,7 +160,7 @@ __global__ void __launch_bounds__(256, TR == 8 ? 2 : TR == 4 ? 3 : 2)
 #pragma unroll
   for (int i = 0; i < TR; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) part[(ty + 8 * i) * kPadW + tx + 8 * j] = acc[i][j];
+    for (int j = 0; j < TC; ++j) part[(ty + 8 * i) * kPadW + tx + 8 * j] = acc[i][j];
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < kTM * kTN / 256; ++q) {
@@ -212,15 +211,29 @@ __global__ void __launch_bounds__(32 * kF64Warps) k_net_f64_layer(const float* _
 }  // namespace
 
 namespace {
-template <int TR, int ST, bool V4>
-cudaError_t net_layer(const float* a, int64_t lda, int32_t count, const float* W, const float* b, int32_t fi,
-                      int32_t fo, int32_t ak, float* o, int64_t ldo, cudaStream_t s) {
-  using Tile = NetTile<TR, ST>;
-  const cudaError_t e = ensure_smem_limit<k_net_layer<TR, ST, V4>>(Tile::kSmem);
+struct NetLaunch {
+  const float* a;
+  int64_t lda;
+  int32_t count;
+  const float *W, *b;
+  int32_t fi, fo, ak;
+  float* o;
+  int64_t ldo;
+};
+
+template <int TR, int TC, int ST, bool V4>
+cudaError_t net_layer(const NetLaunch& n, cudaStream_t s) {
+  using Tile = NetTile<TR, TC, ST>;
+  const cudaError_t e = ensure_smem_limit<k_net_layer<TR, TC, ST, V4>>(Tile::kSmem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_net_layer<TR, ST, V4>,
-                    dim3((unsigned)((count + Tile::kTM - 1) / Tile::kTM), (unsigned)((fo + kTN - 1) / kTN)), dim3(256),
-                    Tile::kSmem, s, a, lda, count, W, b, fi, fo, ak, o, ldo);
+  const dim3 grid((unsigned)((n.count + Tile::kTM - 1) / Tile::kTM), (unsigned)((n.fo + Tile::kTN - 1) / Tile::kTN));
+  return launch_pdl(k_net_layer<TR, TC, ST, V4>, grid, dim3(256), Tile::kSmem, s, n.a, n.lda, n.count, n.W, n.b, n.fi,
+                    n.fo, n.ak, n.o, n.ldo);
+}
+
+template <int TR, int TC, int ST>
+cudaError_t net_layer(const NetLaunch& n, bool v4, cudaStream_t s) {
+  return v4 ? net_layer<TR, TC, ST, true>(n, s) : net_layer<TR, TC, ST, false>(n, s);
 }
 }  // namespace
 
@@ -232,20 +245,25 @@ int launch_net_layer(const float* a, int64_t lda, int32_t count, const float* W,
     return -1;
   // 16-byte copies where every row of both operands starts on 16 bytes (a
   // chunk starts at a multiple of 16, and k % 4 == 0 makes its end whole)
-  const bool v4 = fi % 4 == 0 && lda % 4 == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(W)) & 15u) == 0;
-  // 64-row tiles where they fill the SMs, else 32-row tiles where those do,
-  // else 8-row tiles with eight slabs in flight (few rows: latency-bound)
-  const int64_t cols = (fo + kTN - 1) / kTN;
+  const bool v4 = fi % 4 == 0 && lda % 4 == 0 &&
+                  ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(W)) & 15u) == 0;
+  const NetLaunch n = {a, lda, count, W, b, fi, fo, ak, o, ldo};
+  auto blocks = [&](int tm, int tn) { return (int64_t)((count + tm - 1) / tm) * ((fo + tn - 1) / tn); };
+  // Tiles of 64 x 64 where they occupy most SMs (a thread's 16 shared loads
+  // then serve 256 FMAs, 12 serve 128 with 64 x 32, and the width of those
+  // loads bounds the multiply: 1,000 x 512 x 512 22.5 us with 64 x 32, 20.6 us
+  // with 64 x 64, caches cold), else the widest tile that fills the SMs; with
+  // few rows 8-row tiles with eight slabs in flight (latency-bound: 40 x 512 x
+  // 512 11.2 us with 32-row tiles, 7.2 us with these).
   cudaError_t e;
-  if ((int64_t)((count + 63) / 64) * cols >= sms)
-    e = v4 ? net_layer<8, 3, true>(a, lda, count, W, b, fi, fo, ak, o, ldo, s)
-           : net_layer<8, 3, false>(a, lda, count, W, b, fi, fo, ak, o, ldo, s);
-  else if ((int64_t)((count + 31) / 32) * cols >= sms)
-    e = v4 ? net_layer<4, 3, true>(a, lda, count, W, b, fi, fo, ak, o, ldo, s)
-           : net_layer<4, 3, false>(a, lda, count, W, b, fi, fo, ak, o, ldo, s);
+  if (4 * blocks(64, 64) >= 3 * sms)
+    e = net_layer<8, 8, 4>(n, v4, s);
+  else if (blocks(64, 32) >= sms)
+    e = net_layer<8, 4, 3>(n, v4, s);
+  else if (blocks(32, 32) >= sms)
+    e = net_layer<4, 4, 3>(n, v4, s);
   else
-    e = v4 ? net_layer<1, 8, true>(a, lda, count, W, b, fi, fo, ak, o, ldo, s)
-           : net_layer<1, 8, false>(a, lda, count, W, b, fi, fo, ak, o, ldo, s);
+    e = net_layer<1, 4, 8>(n, v4, s);
   return e == cudaSuccess ? 1 : -1;
 }
 
