@@ -33,6 +33,8 @@ struct TcPlan {
   int tuned = 0;            // pair kernel: 1 if the tile shape and depth were chosen by timing
   int ktail = 0;            // pair kernel: MMAs of the partial last K atom taken through the K-tail buffers
                             // (their shared memory is reserved), 0 = the atom is a pipeline stage of its own
+  int priority = 0;         // pair kernel: launch priority (0: the stream's)
+  int64_t partial_stride = 0;  // pair kernel: columns of `partial` (0: the launch's count)
   const void* w_base = nullptr;  // pair kernel: the first-layer operand and its rows (for re-encoding W1's maps)
   int64_t w_rows = 0;
 };
@@ -73,6 +75,7 @@ int launch_fitness_tc(const TcPlan& plan, const Mlp& mlp, int64_t first, const f
 // Arguments of one launch of the CTA-pair kernel (one handle's rows).
 struct PairArgs {
   int32_t count;        // sparks in this launch
+  int32_t stride;       // columns of `partial` (>= count)
   int32_t first_spark;  // first spark row of the launch (operand tensor maps)
   int32_t m_pairs;      // 256-sample tiles
   int32_t m_tiles;      // 128-sample tiles (rows of `partial`)
@@ -96,7 +99,7 @@ struct PairArgs {
   int64_t bl_off;       // the logits' bias
   const float* rows;    // FP32 spark rows of this launch (biases)
   const int32_t* y;
-  float* partial;       // [m_tiles][count]
+  float* partial;       // [m_tiles][stride]
   uint32_t* status;
   uint64_t wait_budget; // clock64 ticks before a wait gives up (0 = the default)
 };

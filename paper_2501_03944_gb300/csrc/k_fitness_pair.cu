@@ -673,7 +673,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads(S), 1)
       if (et < prev.s_valid && m128 < m.m_tiles) {
         const int s = et;
         const float v = ((red[s * 4 + 0] + red[s * 4 + 1]) + red[s * 4 + 2]) + red[s * 4 + 3];
-        m.partial[(int64_t)m128 * m.count + prev.s0 + s] = v;
+        m.partial[(int64_t)m128 * m.stride + prev.s0 + s] = v;
       }
       prev.on = false;
     };
@@ -791,7 +791,7 @@ cudaError_t launch_pair(const TcPlan& plan, const PairArgs& args, cudaStream_t s
   }
   const int tiles = args.m_pairs * args.n_tiles;
   const int pairs = tiles < plan.pairs ? tiles : plan.pairs;
-  return launch_pdl(k_fitness_pair<H1, H2, NL, S, F8, false>, dim3(2 * pairs), dim3(pair_threads(S)),
+  return launch_pdl_at(plan.priority, k_fitness_pair<H1, H2, NL, S, F8, false>, dim3(2 * pairs), dim3(pair_threads(S)),
                     plan.smem_bytes, s, plan.tmap_x3, plan.tmap_x, plan.tmap_wk, plan.tmap_w, plan.tmap_w2b,
                     plan.tmap_w3b, plan.tmap_xt, plan.tmap_wt, args, static_cast<const PairMember*>(nullptr), 0);
 }
@@ -838,6 +838,7 @@ PairArgs make_args(const TcPlan& plan, const Mlp& mlp, int64_t first, const floa
   const int S = plan.sparks_per_tile;
   const bool l3 = mlp.n_layers == 3;
   a.count = count;
+  a.stride = plan.partial_stride > 0 ? (int32_t)plan.partial_stride : count;
   a.first_spark = (int32_t)first;
   a.m_pairs = (int32_t)((mlp.N + 2 * kPM - 1) / (2 * kPM));
   a.m_tiles = (int32_t)((mlp.N + kPM - 1) / kPM);

@@ -113,8 +113,9 @@ __device__ __forceinline__ float signed_u24(uint32_t r) {
   return __fmaf_rn(__uint2float_rn(r >> 8), 0x1p-23f, -1.0f);
 }
 
-// grid (coordinate blocks, lambda, B * mu): one block covers kExplodeBlocks *
-// kThreads Philox blocks (4 coordinates each) of one spark row; each thread
+// grid (coordinate blocks, rows y, z): spark row row0 + z gridDim.y + y; one
+// block covers kExplodeBlocks * kThreads Philox blocks (4 coordinates each) of
+// one spark row; each thread
 // takes kExplodeBlocks of them, kThreads apart, so a warp's stores stay
 // contiguous.  Global firework z = b * mu + i, spark row z * lam + j, Philox
 // unit (i + fw_off) * lam + j of run b's stream.  The thread's firework
@@ -198,14 +199,15 @@ __device__ __forceinline__ void explode_blocks(const Problem& p, const PhiloxKey
 __global__ void __launch_bounds__(kThreads) k_explode(Problem p, const uint32_t* __restrict__ gens_done,
                                                       const float* __restrict__ fw_x,
                                                       const float* __restrict__ fw_amp,
-                                                      float* __restrict__ sparks, const OpDesc op) {
+                                                      float* __restrict__ sparks, const OpDesc op,
+                                                      const uint32_t row0) {
   griddep_wait();
   griddep_launch_dependents();
   const uint32_t gen = *gens_done + 1u;  // this generation (the counter is advanced by the selection)
-  const uint32_t z = blockIdx.z;
+  const uint32_t row = row0 + blockIdx.z * gridDim.y + blockIdx.y;
+  const uint32_t z = row / (uint32_t)p.lam, j = row - z * (uint32_t)p.lam;
   const uint32_t b = z / (uint32_t)p.mu, i = z - b * (uint32_t)p.mu;
-  const uint32_t row = z * (uint32_t)p.lam + blockIdx.y;
-  const uint32_t unit = (i + (uint32_t)p.fw_off) * (uint32_t)p.lam + blockIdx.y;
+  const uint32_t unit = (i + (uint32_t)p.fw_off) * (uint32_t)p.lam + j;
   uint32_t k0, k1;
   run_key(p, (int)b, k0, k1);
   const PhiloxKeys rk = philox_keys(k0, k1);  // shared by the thread's Philox blocks
@@ -377,9 +379,11 @@ int launch_init(const Problem& p, float* fw_x, float* fw_amp, cudaStream_t s) {
 }
 
 int launch_explode(const Problem& p, const uint32_t* gens_done, const float* fw_x, const float* fw_amp, float* sparks,
-                   const OpDesc& op, cudaStream_t s) {
-  dim3 grid((unsigned)((p.Dp / 4 + kExplodeBlocks * kThreads - 1) / (kExplodeBlocks * kThreads)), p.lam, p.B * p.mu);
-  return launch_pdl(k_explode, grid, dim3(kThreads), 0, s, p, gens_done, fw_x, fw_amp, sparks, op) == cudaSuccess
+                   const OpDesc& op, cudaStream_t s, int64_t row0, int32_t rows) {
+  const unsigned x = (unsigned)((p.Dp / 4 + kExplodeBlocks * kThreads - 1) / (kExplodeBlocks * kThreads));
+  const dim3 grid = rows > 0 ? dim3(x, (unsigned)rows) : dim3(x, p.lam, p.B * p.mu);
+  return launch_pdl(k_explode, grid, dim3(kThreads), 0, s, p, gens_done, fw_x, fw_amp, sparks, op, (uint32_t)row0) ==
+                 cudaSuccess
              ? 1
              : -1;
 }

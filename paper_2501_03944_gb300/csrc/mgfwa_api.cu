@@ -442,6 +442,75 @@ mgfwa_status run_phase(mgfwa_t* h, int32_t phase) {
   return fail(h, MGFWA_EINVAL, "unknown phase %d", phase);
 }
 
+// Fewest waves of the pair kernel's grid to a chunk, and the most chunks: the
+// first chunk's sampling is not hidden, each launch costs its start and end.
+// Measured, a generation whole / in chunks: 3072-128-64-10 BF16 (215 waves)
+// 6,135 / 5,879 us (2), 5,739 (6), 5,738 (8); E4M3 4,316 / 3,947 (8); 784-128-10
+// BF16 (108 waves) 1,185 / 1,151 (2), 1,166 (4); E4M3 (54 waves) 545 / 547 (2).
+constexpr int kOverlapWaves = 30, kOverlapMax = 8;
+
+// Tiles per explosion chunk of an overlapped generation (0: the generation is
+// not overlapped).  A chunk is whole waves of the pair kernel's persistent
+// grid, so that splitting the launch adds no partly filled wave.
+int32_t overlap_tiles(const mgfwa_t* h) {
+  if (h->kind != MGFWA_OBJ_MLP_CE || !use_tc(h, h->cfg.precision) || !h->tc.pair || h->cfg.lagged_guiding) return 0;
+  const int64_t n_e = (int64_t)h->p.B * h->p.mu * h->p.lam;
+  const int64_t tiles = (n_e + h->tc.sparks_per_tile - 1) / h->tc.sparks_per_tile;
+  const int32_t m_pairs = (int32_t)((h->mlp.N + 255) / 256);
+  int32_t a = h->tc.pairs, b = m_pairs;
+  while (b != 0) {
+    const int32_t r = a % b;
+    a = b;
+    b = r;
+  }
+  const int64_t unit = h->tc.pairs / a;  // n-tiles of a whole number of waves
+  // the 320-thread instances (two sparks a tile) leave registers for three
+  // sampler blocks per SM, the larger ones for one or two, beside which the
+  // sampler is too slow to gain anything (784-64-10: 366 us a generation
+  // whole, 378 in two chunks)
+  if (h->tc.sparks_per_tile > 2) return 0;
+  const int64_t waves = tiles * m_pairs / h->tc.pairs;
+  const int64_t chunks = waves / kOverlapWaves < kOverlapMax ? waves / kOverlapWaves : kOverlapMax;
+  if (chunks < 2) return 0;
+  const int64_t per = (tiles / chunks + unit - 1) / unit * unit;
+  if (per >= tiles || per * h->tc.sparks_per_tile > 65535) return 0;
+  return (int32_t)per;
+}
+
+// The explosion and its evaluation, chunk by chunk: chunk c + 1 is drawn on
+// `side` while the pair kernel evaluates chunk c on the handle's stream.  The
+// sampler is bound by integer arithmetic and writes, the pair kernel by the
+// tensor cores, and the pair kernel's one CTA per SM leaves registers for a
+// few sampler blocks beside it; its launches have the higher priority, so that
+// its CTAs are placed first.
+mgfwa_status explode_eval_overlapped(mgfwa_t* h, int32_t per, cudaStream_t side, std::vector<cudaEvent_t>& ev) {
+  const Problem& p = h->p;
+  const int64_t n_e = (int64_t)p.B * p.mu * p.lam;
+  h->lag_now = false;
+  int least = 0, greatest = 0;
+  if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess) return cuda_fail(h, "stream priorities");
+  TcPlan tc = h->tc;
+  tc.priority = greatest;
+  tc.partial_stride = n_e;
+  const int64_t chunk = (int64_t)per * h->tc.sparks_per_tile;
+  for (int64_t r0 = 0; r0 < n_e; r0 += chunk) {
+    const int32_t rows = (int32_t)(n_e - r0 < chunk ? n_e - r0 : chunk);
+    MG_LAUNCH(h, launch_explode(p, h->gens_done, h->fw_x, h->fw_amp, h->sparks, op_rows(h, 0),
+                                r0 == 0 ? h->stream : side, r0, rows),
+              "explode");
+    cudaEvent_t e = nullptr;
+    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return cuda_fail(h, "overlap event");
+    ev.push_back(e);
+    if (cudaEventRecord(e, r0 == 0 ? h->stream : side) != cudaSuccess ||
+        cudaStreamWaitEvent(r0 == 0 ? side : h->stream, e, 0) != cudaSuccess)
+      return cuda_fail(h, "overlap order");
+    MG_LAUNCH(h, launch_fitness_tc(tc, h->mlp, r0, h->sparks + r0 * p.Dp, p.Dp, rows, h->op_scale, h->partial + r0,
+                                   h->status, h->stream),
+              "tensor-core fitness");
+  }
+  return MGFWA_OK;
+}
+
 // Capture the phases explode .. select into h->gen_exec, on a private stream
 // swapped in for the handle's (so the caller's stream is never in capture
 // mode).  Nothing in them depends on the host's generation counter: the
@@ -451,13 +520,25 @@ mgfwa_status capture_generation(mgfwa_t* h) {
   if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return cuda_fail(h, "capture stream");
   cudaStream_t own = h->stream;
   const int64_t before = h->launches;
+  const int32_t per = overlap_tiles(h);
+  cudaStream_t side = nullptr;
+  std::vector<cudaEvent_t> ev;
+  if (per > 0 && cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaStreamDestroy(cs);
+    return cuda_fail(h, "capture side stream");
+  }
   cudaGraph_t graph = nullptr;
   mgfwa_status st = MGFWA_OK;
   bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   if (ok) {
     h->stream = cs;
     h->capturing = true;
-    for (int32_t ph = MGFWA_PHASE_EXPLODE; ph <= MGFWA_PHASE_SELECT && st == MGFWA_OK; ++ph) st = run_phase(h, ph);
+    int32_t ph = MGFWA_PHASE_EXPLODE;
+    if (per > 0) {
+      st = explode_eval_overlapped(h, per, side, ev);
+      ph = MGFWA_PHASE_RANK;
+    }
+    for (; ph <= MGFWA_PHASE_SELECT && st == MGFWA_OK; ++ph) st = run_phase(h, ph);
     h->capturing = false;
     h->stream = own;
     ok = cudaStreamEndCapture(cs, &graph) == cudaSuccess && st == MGFWA_OK;
@@ -469,6 +550,8 @@ mgfwa_status capture_generation(mgfwa_t* h) {
     if (st == MGFWA_OK) st = cuda_fail(h, "generation graph capture");
   }
   if (graph) cudaGraphDestroy(graph);
+  for (cudaEvent_t e : ev) cudaEventDestroy(e);
+  if (side) cudaStreamDestroy(side);
   cudaStreamDestroy(cs);
   return st;
 }

@@ -118,20 +118,28 @@ __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// launch_pdl_at: with a launch priority (0: the stream's).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                              Args... args) {
+inline cudaError_t launch_pdl_at(int priority, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                 cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePriority;
+  attr[1].val.priority = priority;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = priority != 0 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              Args... args) {
+  return launch_pdl_at(0, kernel, grid, block, smem, s, args...);
 }
 
 // Raise kernel K's dynamic shared-memory limit on the current device once.
@@ -255,9 +263,10 @@ int launch_init(const Problem& p, float* fw_x, float* fw_amp, cudaStream_t s);
 // non-null also the BF16 first-layer operand (w1_elems per spark row).
 // The generation number is read on the device: gens_done[0] + 1, where
 // gens_done counts completed generations (launch_select advances it), so a
-// captured generation replays with the right Philox counters.
+// captured generation replays with the right Philox counters.  With rows > 0
+// (at most 65535) only the spark rows [row0, row0 + rows) are made.
 int launch_explode(const Problem& p, const uint32_t* gens_done, const float* fw_x, const float* fw_amp,
-                   float* sparks, const OpDesc& op, cudaStream_t s);
+                   float* sparks, const OpDesc& op, cudaStream_t s, int64_t row0 = 0, int32_t rows = 0);
 
 // With `partial` ([mtiles][stride] per-sample-tile loss sums, the explosion
 // rows first, N samples; stride 0 means B*mu*lam), the rank kernel also
