@@ -47,6 +47,7 @@ struct Bars {
   uint64_t full[kMaxStages];   // stage landed (TMA)
   uint64_t empty[kMaxStages];  // stage free (its MMAs completed)
   uint64_t done;
+  uint64_t read;               // k_net_x3: the epilogue has read a split's accumulators
   uint32_t tmem_base;
   volatile int abort_flag;
 };
@@ -622,10 +623,12 @@ int launch_l1_fp32x3(const L1Plan& pl, const Mlp& mlp, const int32_t* idx, int32
 // weights W are both given as three BF16 parts, the same six products and
 // three accumulators as above.  One CTA per 128 rows x 128 outputs x one
 // K split of kNetKPer 32-element blocks (splits = ceil(fan_in / 128): a
-// number fixed by the layer's fan-in alone).  Up to kNetCluster splits of a
-// tile form a thread-block cluster: each CTA leaves its partial sum ((even +
-// odd) + corrections) in its shared memory, and after a cluster barrier the
-// CTAs share the tile's columns, each adding the partials of its columns in
+// number fixed by the layer's fan-in alone), or two splits one after the other
+// where there are more than kNetOne (1,040 x 512 x 1000: eight CTAs of one
+// split to a cluster 36 us, the clusters of eight taking three waves).  Up to
+// 2 kNetCluster splits of a tile form a thread-block cluster: each CTA leaves
+// its splits' partial sums ((even + odd) + corrections) in its shared memory,
+// and after a cluster barrier the CTAs share the tile's columns, each adding the partials of its columns in
 // split order through distributed shared memory, then the bias and the
 // activation, and writing the FP32 output and/or its three BF16 parts (the
 // next tensor-core layer's A).  With more splits the partials go to memory
@@ -635,23 +638,28 @@ int launch_l1_fp32x3(const L1Plan& pl, const Mlp& mlp, const int32_t* idx, int32
 //
 // At 1,040 rows a 512 x 512 layer is 36 tiles x 4 splits: its six products
 // take about 1 us of tensor time, so what bounds it is the latency of one
-// pass -- loads, MMAs, epilogue, the sum -- and the traffic around it.  All
-// of a CTA's K blocks are in flight at once (no ring), the weights' before
-// the previous layer has finished.
+// pass -- loads, MMAs, epilogue, the sum -- and the traffic around it.  All of
+// one split's K blocks are in flight at once, the first weights' before the
+// previous layer has finished.  Measured at that size (launch list, caches
+// cold): 17.6 us and 6.7 us for the sum as a kernel of its own, 13.0 us so.
 
 namespace {
 
 constexpr int kNetKPer = 4;      // 32-element K blocks per split
-constexpr int kNetCluster = 8;   // splits of a tile that meet in one cluster (the portable size)
+constexpr int kNetCluster = 8;   // CTAs of a cluster at most (the portable size)
+constexpr int kNetOne = 4;       // splits up to this: one to a CTA; above, two
 constexpr int kNetThreads = 320; // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue (two per TMEM lane quadrant)
-static_assert(kNetKPer <= kStages, "every K block of a split has its own stage");
-static_assert((size_t)kBM * kN * sizeof(float) <= (size_t)kStages * kStageBytes, "partial tile fits in the stages");
+constexpr int kNetRing = 3;      // stages with two splits to a CTA
+constexpr size_t kNetTile = (size_t)kBM * kN * sizeof(float);  // one split's partial tile
+static_assert(kNetKPer <= kStages, "every K block of a CTA's one split has its own stage");
+static_assert(kNetTile <= (size_t)kNetRing * kStageBytes, "a partial tile fits in the stages");
 
 struct NetX3Args {
   int32_t rows;        // rows of this launch (A rows [0, rows))
   int32_t k_blocks;    // 32-element K blocks of the fan-in
-  int32_t splits;      // K splits (gridDim.z)
-  float* partial;      // splits > kNetCluster: partial sums [splits][rows][n]; else null
+  int32_t splits;      // K splits
+  int32_t per;         // splits to a CTA (1 or 2; gridDim.z = ceil(splits / per))
+  float* partial;      // more splits than a cluster takes: partial sums [splits][rows][n]; else null
   int32_t n;           // fan-out
   int32_t act;         // activation, or < 0 for none
   const float* bias;   // [n]
@@ -685,6 +693,11 @@ __device__ __forceinline__ float ld_cluster(uint32_t addr) {
   float v;
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
   return v;
+}
+
+// Bytes of a CTA's stages and partial tiles.
+__host__ __device__ __forceinline__ size_t net_x3_data(int per) {
+  return per == 1 ? (size_t)kStages * kStageBytes : (size_t)kNetRing * kStageBytes + kNetTile;
 }
 
 // Outputs col .. col + 7 of row r (z: the sums with the bias not yet added):
@@ -732,16 +745,25 @@ __global__ void __launch_bounds__(kNetThreads, 1)
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   auto Ap = [&](int p, int s) { return base + ((size_t)s * 2 * kParts + p) * kPartBytes; };
   auto Wp = [&](int p, int s) { return base + ((size_t)s * 2 * kParts + kParts + p) * kPartBytes; };
-  Bars* sb = reinterpret_cast<Bars*>(base + (size_t)kStages * kStageBytes);
-  float* part = reinterpret_cast<float*>(base);  // the split's partial tile [column][row], once the MMAs are done
+  const int S = a.per == 1 ? kStages : kNetRing;
+  // local split i's partial tile [column][row]: the CTA's last one in the stages, once its MMAs are done; with two
+  // to a CTA the first one behind them
+  float* const tile_last = reinterpret_cast<float*>(base);
+  float* const tile_first = a.per == 1 ? tile_last : reinterpret_cast<float*>(base + (size_t)kNetRing * kStageBytes);
+  Bars* sb = reinterpret_cast<Bars*>(base + net_x3_data(a.per));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mt = blockIdx.x, nt = blockIdx.y;
-  // this CTA's K blocks [kb0, kb0 + nkb)
-  const int kb0 = (int)blockIdx.z * kNetKPer;
-  const int nkb = min(kNetKPer, a.k_blocks - kb0);
+  // this CTA's splits and K blocks [kb0, kb0 + nkb)
+  const int sp0 = (int)blockIdx.z * a.per, nsp = min(a.per, a.splits - sp0);
+  const int kb0 = sp0 * kNetKPer;
+  const int nkb = min(nsp * kNetKPer, a.k_blocks - kb0);
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(&sb->full[s], 1);
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&sb->full[s], 1);
+      mbar_init(&sb->empty[s], 1);
+    }
     mbar_init(&sb->done, 1);
+    mbar_init(&sb->read, kNetThreads / 32 - 2);
     sb->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -757,48 +779,75 @@ __global__ void __launch_bounds__(kNetThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = sb->tmem_base;
 
+  auto load_w = [&](int kb) {
+#pragma unroll
+    for (int p = 0; p < kParts; ++p)
+      tma_3d(Wp(p, kb % S), &tmap_w, (kb0 + kb) * kBKf, nt * kN, p, &sb->full[kb % S]);
+  };
+  auto load_a = [&](int kb) {
+#pragma unroll
+    for (int p = 0; p < kParts; ++p)
+      tma_3d(Ap(p, kb % S), &tmap_a, (kb0 + kb) * kBKf, mt * kBM, p, &sb->full[kb % S]);
+  };
   // The weights' parts were written when the handle was made: their copies
   // start before the previous kernel (the layer's input) has finished.
+  const int first = min(nkb, S);
   if (warp == 0 && lane == 0) {
-    for (int kb = 0; kb < nkb; ++kb) {
+    for (int kb = 0; kb < first; ++kb) {
       mbar_expect_tx(&sb->full[kb], kStageBytes);
-#pragma unroll
-      for (int p = 0; p < kParts; ++p) tma_3d(Wp(p, kb), &tmap_w, (kb0 + kb) * kBKf, nt * kN, p, &sb->full[kb]);
+      load_w(kb);
     }
   }
   griddep_wait();
   griddep_launch_dependents();
   if (warp == 0) {
     if (lane == 0) {
-      for (int kb = 0; kb < nkb; ++kb)
-#pragma unroll
-        for (int p = 0; p < kParts; ++p) tma_3d(Ap(p, kb), &tmap_a, (kb0 + kb) * kBKf, mt * kBM, p, &sb->full[kb]);
+      for (int kb = 0; kb < first; ++kb) load_a(kb);
+      int kb = first;
+      for (; kb < nkb; ++kb) {
+        if (!mbar_wait(sb, &sb->empty[kb % S], (uint32_t)(kb / S - 1) & 1u, a.status, 1u)) break;
+        mbar_expect_tx(&sb->full[kb % S], kStageBytes);
+        load_w(kb);
+        load_a(kb);
+      }
       // every issued copy lands before the CTA may exit
-      for (int kb = 0; kb < nkb; ++kb) mbar_drain(&sb->full[kb], 0u, a.status);
+      for (int j = kb - S > 0 ? kb - S : 0; j < kb; ++j)
+        mbar_drain(&sb->full[j % S], (uint32_t)(j / S) & 1u, a.status);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16(kBM, kN);
-      for (int kb = 0; kb < nkb; ++kb) {
-        if (!mbar_wait(sb, &sb->full[kb], 0u, a.status, 2u)) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t x1 = smem_u32(Ap(0, kb)), x2 = smem_u32(Ap(1, kb)), x3 = smem_u32(Ap(2, kb));
-        const uint32_t w1 = smem_u32(Wp(0, kb)), w2 = smem_u32(Wp(1, kb)), w3 = smem_u32(Wp(2, kb));
-        const uint32_t d_main = tmem + (uint32_t)((kb & 1) * kN), d_corr = tmem + (uint32_t)(2 * kN);
+      bool ok = true;
+      for (int i = 0; i < nsp; ++i) {
+        // the accumulators are free once the epilogue has read the split before
+        if (ok && i > 0) ok = mbar_wait(sb, &sb->read, (uint32_t)(i - 1) & 1u, a.status, 4u);
+        const int k1 = min((i + 1) * kNetKPer, nkb);
+        for (int kb = i * kNetKPer; ok && kb < k1; ++kb) {
+          const int s = kb % S, l = kb - i * kNetKPer;  // l: block of the split
+          if (!mbar_wait(sb, &sb->full[s], (uint32_t)(kb / S) & 1u, a.status, 2u)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t x1 = smem_u32(Ap(0, s)), x2 = smem_u32(Ap(1, s)), x3 = smem_u32(Ap(2, s));
+          const uint32_t w1 = smem_u32(Wp(0, s)), w2 = smem_u32(Wp(1, s)), w3 = smem_u32(Wp(2, s));
+          const uint32_t d_main = tmem + (uint32_t)((l & 1) * kN), d_corr = tmem + (uint32_t)(2 * kN);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const uint32_t o = (uint32_t)j * 32u;
-          const uint32_t first = (kb < 2 && j == 0) ? 0u : 1u;
-          const uint32_t first_c = (kb == 0 && j == 0) ? 0u : 1u;
-          mma_bf16(d_main, smem_desc_sw64(x1 + o), smem_desc_sw64(w1 + o), idesc, first);
-          mma_bf16(d_corr, smem_desc_sw64(x1 + o), smem_desc_sw64(w2 + o), idesc, first_c);
-          mma_bf16(d_corr, smem_desc_sw64(x2 + o), smem_desc_sw64(w1 + o), idesc, 1u);
-          mma_bf16(d_corr, smem_desc_sw64(x2 + o), smem_desc_sw64(w2 + o), idesc, 1u);
-          mma_bf16(d_corr, smem_desc_sw64(x1 + o), smem_desc_sw64(w3 + o), idesc, 1u);
-          mma_bf16(d_corr, smem_desc_sw64(x3 + o), smem_desc_sw64(w1 + o), idesc, 1u);
+          for (int j = 0; j < 2; ++j) {
+            const uint32_t o = (uint32_t)j * 32u;
+            const uint32_t first_m = (l < 2 && j == 0) ? 0u : 1u;
+            const uint32_t first_c = (l == 0 && j == 0) ? 0u : 1u;
+            mma_bf16(d_main, smem_desc_sw64(x1 + o), smem_desc_sw64(w1 + o), idesc, first_m);
+            mma_bf16(d_corr, smem_desc_sw64(x1 + o), smem_desc_sw64(w2 + o), idesc, first_c);
+            mma_bf16(d_corr, smem_desc_sw64(x2 + o), smem_desc_sw64(w1 + o), idesc, 1u);
+            mma_bf16(d_corr, smem_desc_sw64(x2 + o), smem_desc_sw64(w2 + o), idesc, 1u);
+            mma_bf16(d_corr, smem_desc_sw64(x1 + o), smem_desc_sw64(w3 + o), idesc, 1u);
+            mma_bf16(d_corr, smem_desc_sw64(x3 + o), smem_desc_sw64(w1 + o), idesc, 1u);
+          }
+          if (kb + S < nkb) mma_commit(&sb->empty[s]);
         }
+        mma_commit(&sb->done);  // after every issued MMA (also on abort)
       }
-      mma_commit(&sb->done);  // after every issued MMA (also on abort)
     }
   }
   const int q = warp & 3, half = (warp - 2) >> 2;  // epilogue warps: TMEM lane quadrant, half of the columns
@@ -807,30 +856,39 @@ __global__ void __launch_bounds__(kNetThreads, 1)
   const bool inside = r < a.rows;
   if (warp >= 2) {
     const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
-    mbar_drain(&sb->done, 0u, a.status);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const bool odd = nkb > 1;
+    for (int sp = 0; sp < nsp; ++sp) {
+      mbar_drain(&sb->done, (uint32_t)sp & 1u, a.status);
+      __syncwarp();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      float* part = sp == 0 ? tile_first : tile_last;
+      const bool odd = min(kNetKPer, nkb - sp * kNetKPer) > 1;
 #pragma unroll 1
-    for (int j0 = half * (kN / 2); j0 < (half + 1) * (kN / 2); j0 += 16) {
-      float x[16], x1[16], xc[16];
+      for (int j0 = half * (kN / 2); j0 < (half + 1) * (kN / 2); j0 += 16) {
+        float x[16], x1[16], xc[16];
 #pragma unroll
-      for (int h = 0; h < 16; h += 8) {
-        tmem_ld8(lanes + (uint32_t)(j0 + h), x + h);
-        tmem_ld8(lanes + (uint32_t)(kN + j0 + h), x1 + h);
-        tmem_ld8(lanes + (uint32_t)(2 * kN + j0 + h), xc + h);
+        for (int h = 0; h < 16; h += 8) {
+          tmem_ld8(lanes + (uint32_t)(j0 + h), x + h);
+          tmem_ld8(lanes + (uint32_t)(kN + j0 + h), x1 + h);
+          tmem_ld8(lanes + (uint32_t)(2 * kN + j0 + h), xc + h);
+        }
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] = (odd ? x[i] + x1[i] : x[i]) + xc[i];
+        if (!a.partial) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) part[(j0 + i) * kBM + rrow] = x[i];
+        } else if (inside && !sb->abort_flag) {
+          const int col = nt * kN + j0;
+          float* prow = a.partial + ((int64_t)(sp0 + sp) * a.rows + r) * a.n + col;
+#pragma unroll
+          for (int i = 0; i < 16; i += 2)
+            if (col + i < a.n) *reinterpret_cast<float2*>(prow + i) = make_float2(x[i], x[i + 1]);
+        }
       }
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-      for (int i = 0; i < 16; ++i) x[i] = (odd ? x[i] + x1[i] : x[i]) + xc[i];
-      if (!a.partial) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) part[(j0 + i) * kBM + rrow] = x[i];
-      } else if (inside && !sb->abort_flag) {
-        const int col = nt * kN + j0;
-        float* prow = a.partial + ((int64_t)blockIdx.z * a.rows + r) * a.n + col;
-#pragma unroll
-        for (int i = 0; i < 16; i += 2)
-          if (col + i < a.n) *reinterpret_cast<float2*>(prow + i) = make_float2(x[i], x[i + 1]);
+      if (sp + 1 < nsp) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sb->read);
       }
     }
   }
@@ -841,14 +899,16 @@ __global__ void __launch_bounds__(kNetThreads, 1)
     if (warp >= 2) {
       // this CTA's columns of the tile, eight at a time: the cluster's partials in split order
       const bool store = inside && !sb->abort_flag;
-      for (int o = (int)cluster_rank() + a.splits * half; o < kN / 8; o += 2 * a.splits) {
+      const int ctas = (int)gridDim.z;
+      for (int o = (int)cluster_rank() + ctas * half; o < kN / 8; o += 2 * ctas) {
         const int col = nt * kN + o * 8;
         if (col >= a.n) break;
-        const uint32_t at = smem_u32(part + o * 8 * kBM + rrow);
+        const uint32_t at0 = smem_u32(tile_first + o * 8 * kBM + rrow), at1 = smem_u32(tile_last + o * 8 * kBM + rrow);
         float z[8];
 #pragma unroll 4
         for (int sp = 0; sp < a.splits; ++sp) {
-          const uint32_t peer = map_to(at, (uint32_t)sp);
+          const int c = a.per == 1 ? sp : sp >> 1;
+          const uint32_t peer = map_to(sp == c * a.per ? at0 : at1, (uint32_t)c);
           float v[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) v[i] = ld_cluster(peer + (uint32_t)(i * kBM * (int)sizeof(float)));
@@ -927,7 +987,11 @@ cudaError_t launch_pdl_z(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-size_t net_x3_smem() { return 1024 + (size_t)kStages * kStageBytes + ((sizeof(Bars) + 15) & ~size_t(15)) + 64; }
+size_t net_x3_smem(int per) { return 1024 + net_x3_data(per) + ((sizeof(Bars) + 15) & ~size_t(15)) + 64; }
+
+// Splits to a CTA, and whether a tile's CTAs fit a cluster.
+int net_x3_per(int splits) { return splits > kNetOne && splits <= 2 * kNetCluster ? 2 : 1; }
+bool net_x3_clustered(int splits) { return splits <= 2 * kNetCluster; }
 
 }  // namespace
 
@@ -941,7 +1005,7 @@ int64_t net_x3_words(const NetOut& net, int64_t max_rows) {
   for (int l = 0; l < net.n_layers; ++l)
     if (net_x3_layer(net.widths[l], net.widths[l + 1]) && net_x3_splits(net.widths[l]) > ks)
       ks = net_x3_splits(net.widths[l]);
-  if (ks > kNetCluster) w += (int64_t)ks * max_rows * net.wmax;  // FP32 partial sums
+  if (!net_x3_clustered(ks)) w += (int64_t)ks * max_rows * net.wmax;  // FP32 partial sums
   for (int l = 0; l < net.n_layers; ++l)
     if (net_x3_layer(net.widths[l], net.widths[l + 1])) w += 3 * (int64_t)net.widths[l + 1] * (net.widths[l] / 2);
   return w;
@@ -965,7 +1029,7 @@ bool net_x3_plan(NetX3Plan& pl, const NetOut& net, int64_t max_rows, uint32_t* b
   for (int l = 0; l < net.n_layers; ++l)
     if (net_x3_layer(net.widths[l], net.widths[l + 1]) && net_x3_splits(net.widths[l]) > ks)
       ks = net_x3_splits(net.widths[l]);
-  if (ks > kNetCluster) {
+  if (!net_x3_clustered(ks)) {
     pl.partial = reinterpret_cast<float*>(wcur);
     wcur += (int64_t)ks * max_rows * net.wmax;
   }
@@ -992,7 +1056,7 @@ bool net_x3_plan(NetX3Plan& pl, const NetOut& net, int64_t max_rows, uint32_t* b
       if (!encode_bf16(&pl.tmap_w[l], pl.w_parts[l], dims, strides, box)) return false;
     }
   }
-  if (!any || ensure_smem_limit<k_net_x3>(net_x3_smem()) != cudaSuccess) {
+  if (!any || ensure_smem_limit<k_net_x3>(net_x3_smem(2)) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -1042,7 +1106,8 @@ int launch_net_output_x3(const NetX3Plan& pl, const NetOut& net, const float* ro
       x.rows = count;
       x.k_blocks = (fi + kBKf - 1) / kBKf;
       x.splits = net_x3_splits(fi);
-      x.partial = x.splits > kNetCluster ? pl.partial : nullptr;
+      x.per = net_x3_per(x.splits);
+      x.partial = net_x3_clustered(x.splits) ? nullptr : pl.partial;
       x.n = fo;
       x.act = ak;
       x.bias = b;
@@ -1051,8 +1116,9 @@ int launch_net_output_x3(const NetX3Plan& pl, const NetOut& net, const float* ro
       x.parts = next_tc ? pl.act_parts[(l + 1) & 1] : nullptr;
       x.plane_words = pl.max_rows * (fo / 2);
       x.status = status;
-      const dim3 grid((unsigned)((count + kBM - 1) / kBM), (unsigned)((fo + kN - 1) / kN), (unsigned)x.splits);
-      if (launch_pdl_z(k_net_x3, grid, dim3(kNetThreads), net_x3_smem(), x.partial ? 1u : (unsigned)x.splits, s,
+      const dim3 grid((unsigned)((count + kBM - 1) / kBM), (unsigned)((fo + kN - 1) / kN),
+                      (unsigned)((x.splits + x.per - 1) / x.per));
+      if (launch_pdl_z(k_net_x3, grid, dim3(kNetThreads), net_x3_smem(x.per), x.partial ? 1u : grid.z, s,
                        pl.tmap_a[l], pl.tmap_w[l], x) != cudaSuccess)
         return -1;
       ++n;
