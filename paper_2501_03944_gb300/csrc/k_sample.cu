@@ -368,6 +368,18 @@ __global__ void k_f32_to_op(const float* __restrict__ src, int64_t n, int32_t ki
   }
 }
 
+// *top = the bits of the largest |src[e]| that is not a NaN (*top is 0 before):
+// the bits of non-negative floats order as the floats do.
+__global__ void __launch_bounds__(256) k_abs_max(const float* __restrict__ src, int64_t n, uint32_t* top) {
+  uint32_t m = 0;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t u = __float_as_uint(src[e]) & 0x7fffffffu;
+    if (u <= 0x7f800000u && u > m) m = u;
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(top, m);
+}
+
 inline unsigned blocks_for(int64_t n4) { return (unsigned)((n4 + kThreads - 1) / kThreads); }
 
 }  // namespace
@@ -417,6 +429,13 @@ int launch_f32_to_op(const float* src, int64_t n, int32_t kind, float inv_scale,
   if (n <= 0) return 0;
   const unsigned blocks = (unsigned)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
   k_f32_to_op<<<blocks, 256, 0, s>>>(src, n, kind, inv_scale, dst);
+  return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
+}
+
+int launch_abs_max(const float* src, int64_t n, uint32_t* top, cudaStream_t s) {
+  if (n <= 0) return 0;
+  const unsigned blocks = (unsigned)((n + 255) / 256 < 1216 ? (n + 255) / 256 : 1216);
+  k_abs_max<<<blocks, 256, 0, s>>>(src, n, top);
   return cudaPeekAtLastError() == cudaSuccess ? 1 : -1;
 }
 

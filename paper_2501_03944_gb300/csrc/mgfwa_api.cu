@@ -42,7 +42,9 @@ struct mgfwa_handle {
   char* arena = nullptr;
   size_t arena_bytes = 0;
   bool pooled = false;       // the arena came from the library's stream-ordered pool
-  uint64_t fingerprint = 0;  // configuration + objective (checkpoints load only into the same problem)
+  int32_t obj_layers = 0;    // the objective's n_layers as given
+  uint64_t fingerprint = 0;  // configuration + objective (checkpoints load only into the same problem): see
+  bool fingerprinted = false;  // ensure_fingerprint
   // device buffers (carved from the arena)
   float* X = nullptr;
   void* Xop = nullptr;          // [N][d_in] X as the tensor-core operand (BF16 or E4M3)
@@ -765,16 +767,36 @@ void arena_free(mgfwa_t* h) {
 }
 
 // FNV-1a over the configuration (but its budget), the network shape and
-// (every 61st element of) the batch: a checkpoint is refused by a handle of
-// another problem.
-uint64_t problem_fingerprint(const mgfwa_config* cfg, const mgfwa_objective* obj) {
+// (every kPrintStep-th element of) the batch or the parameters: a checkpoint
+// is refused by a handle of another problem.  It is taken from the handle's
+// own copies when a checkpoint is first saved or loaded; taken at create it
+// was most of a create's time (one chain of byte steps through a large X:
+// 3072-128-64-10, N = 4096, 2,823 us a create with it, 1,544 us without).
+constexpr int64_t kPrintStep = 61;
+
+mgfwa_status ensure_fingerprint(mgfwa_t* h) {
+  if (h->fingerprinted) return MGFWA_OK;
   uint64_t f = 1469598103934665603ull;
   auto mix = [&](const void* p, size_t n) {
     const unsigned char* b = static_cast<const unsigned char*>(p);
     for (size_t i = 0; i < n; ++i) f = (f ^ b[i]) * 1099511628211ull;
   };
+  // every kPrintStep-th of n 4-byte elements of a device array
+  auto mix_strided = [&](const void* dev, int64_t n) -> mgfwa_status {
+    const int64_t count = (n + kPrintStep - 1) / kPrintStep;
+    if (count < 1) return MGFWA_OK;
+    uint32_t* g = new (std::nothrow) uint32_t[(size_t)count];
+    if (!g) return fail(h, MGFWA_ENOMEM, "checkpoint: host allocation failed");
+    const cudaError_t e = cudaMemcpy2DAsync(g, sizeof(uint32_t), dev, sizeof(uint32_t) * kPrintStep, sizeof(uint32_t),
+                                            (size_t)count, cudaMemcpyDeviceToHost, h->stream);
+    const bool ok = e == cudaSuccess && cudaStreamSynchronize(h->stream) == cudaSuccess;
+    if (ok) mix(g, sizeof(uint32_t) * (size_t)count);
+    delete[] g;
+    return ok ? MGFWA_OK : cuda_fail(h, "checkpoint: read the problem");
+  };
   // field by field (struct padding is not part of the problem); the budget is
   // left out so that a resumed run may be given a larger one
+  const mgfwa_config* cfg = &h->cfg;
   mix(&cfg->dim, sizeof(cfg->dim));
   mix(&cfg->lb, sizeof(cfg->lb));
   mix(&cfg->ub, sizeof(cfg->ub));
@@ -797,23 +819,25 @@ uint64_t problem_fingerprint(const mgfwa_config* cfg, const mgfwa_objective* obj
   mix(&cfg->lagged_guiding, sizeof(cfg->lagged_guiding));
   mix(&cfg->shard_id, sizeof(cfg->shard_id));
   mix(&cfg->n_shards, sizeof(cfg->n_shards));
-  mix(&obj->kind, sizeof(obj->kind));
-  mix(&obj->n_layers, sizeof(obj->n_layers));
-  if (obj->kind == MGFWA_OBJ_MLP_CE) {
-    mix(obj->widths, sizeof(int32_t) * (size_t)(obj->n_layers + 1));
-    mix(obj->acts, sizeof(int32_t) * (size_t)(obj->n_layers > 1 ? obj->n_layers - 1 : 0));
-    mix(&obj->n_samples, sizeof(obj->n_samples));
-    const int64_t nx = obj->n_samples * (int64_t)obj->widths[0];
-    for (int64_t e = 0; e < nx; e += 61) mix(obj->X + e, sizeof(float));
-    for (int64_t e = 0; e < obj->n_samples; e += 61) mix(obj->y + e, sizeof(int32_t));
-  } else if (obj->kind == MGFWA_OBJ_NET_OUTPUT) {
-    mix(obj->widths, sizeof(int32_t) * (size_t)(obj->n_layers + 1));
-    if (obj->n_layers > 1) mix(obj->acts, sizeof(int32_t) * (size_t)(obj->n_layers - 1));
-    int64_t n = 0;
-    for (int l = 0; l < obj->n_layers; ++l) n += (int64_t)obj->widths[l] * obj->widths[l + 1] + obj->widths[l + 1];
-    for (int64_t e = 0; e < n; e += 61) mix(obj->params + e, sizeof(float));
+  mix(&h->kind, sizeof(h->kind));
+  mix(&h->obj_layers, sizeof(h->obj_layers));
+  mgfwa_status st = MGFWA_OK;
+  if (h->kind == MGFWA_OBJ_MLP_CE) {
+    const Mlp& m = h->mlp;
+    mix(m.widths, sizeof(int32_t) * (size_t)(m.n_layers + 1));
+    mix(m.acts, sizeof(int32_t) * (size_t)(m.n_layers - 1));
+    mix(&m.N, sizeof(m.N));
+    st = mix_strided(h->X, m.N * (int64_t)m.widths[0]);
+    if (st == MGFWA_OK) st = mix_strided(h->y, m.N);
+  } else if (h->kind == MGFWA_OBJ_NET_OUTPUT) {
+    mix(h->net.widths, sizeof(int32_t) * (size_t)(h->net.n_layers + 1));
+    if (h->net.n_layers > 1) mix(h->net.acts, sizeof(int32_t) * (size_t)(h->net.n_layers - 1));
+    st = mix_strided(h->net.params, h->net_count);
   }
-  return f;
+  if (st != MGFWA_OK) return st;
+  h->fingerprint = f;
+  h->fingerprinted = true;
+  return MGFWA_OK;
 }
 
 // Fill the handle's problem description and sizes from a validated
@@ -899,19 +923,9 @@ void plan_handle(mgfwa_t* h, const mgfwa_config* cfg, const mgfwa_objective* obj
     }
     h->net_count = off;
   }
-  h->fingerprint = problem_fingerprint(cfg, obj);
+  h->obj_layers = obj->n_layers;
   h->want_op = obj->kind == MGFWA_OBJ_MLP_CE && (cfg->precision == MGFWA_BF16 || cfg->precision == MGFWA_FP8);
   h->op_kind = !h->want_op ? kOpNone : (cfg->precision == MGFWA_FP8 ? kOpFp8 : kOpBf16);
-  if (h->op_kind == kOpFp8) {
-    // E4M3 scales: X by its largest magnitude, the weights by the box bound
-    // (every coordinate lies in [lb, ub], so no spark exceeds it)
-    float amax = 0.0f;
-    for (int64_t e = 0; e < obj->n_samples * (int64_t)obj->widths[0]; ++e) amax = std::fmax(amax, std::fabs(obj->X[e]));
-    const float bound = std::fmax(std::fabs(cfg->lb), std::fabs(cfg->ub));
-    h->inv_x = amax > 0.0f ? 448.0f / amax : 1.0f;
-    h->inv_w = 448.0f / bound;
-    h->op_scale = (float)(1.0 / ((double)h->inv_x * (double)h->inv_w));
-  }
   h->refine = cfg->refine_every > 0 && obj->kind == MGFWA_OBJ_MLP_CE;
   const bool rescore = h->want_op && cfg->elite_rescore > 0;
   if (h->refine || rescore) {
@@ -1094,6 +1108,20 @@ mgfwa_status mgfwa_create(const mgfwa_config* cfg, const mgfwa_objective* obj, v
     if (cudaMemcpyAsync(h->X, obj->X, sizeof(float) * N * d_in, cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
         cudaMemcpyAsync(h->y, obj->y, sizeof(int32_t) * N, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
       return bail(cuda_fail(h, "copy batch"));
+    if (h->op_kind == kOpFp8) {
+      // E4M3 scales: X by its largest magnitude (found on the device: one host thread took 560 us for 2048 x 784,
+      // most of it reading X), the weights by the box bound (every coordinate lies in [lb, ub], so no spark exceeds it)
+      uint32_t* word = reinterpret_cast<uint32_t*>(h->f64);  // cleared above, not yet in use
+      float amax = 0.0f;
+      CREATE_LAUNCH(launch_abs_max(h->X, N * d_in, word, h->stream), "X magnitude");
+      if (cudaMemcpyAsync(&amax, word, sizeof(amax), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
+          cudaStreamSynchronize(h->stream) != cudaSuccess)
+        return bail(cuda_fail(h, "X magnitude"));
+      const float bound = std::fmax(std::fabs(cfg->lb), std::fabs(cfg->ub));
+      h->inv_x = amax > 0.0f ? 448.0f / amax : 1.0f;
+      h->inv_w = 448.0f / bound;
+      h->op_scale = (float)(1.0 / ((double)h->inv_x * (double)h->inv_w));
+    }
     if (want_op) CREATE_LAUNCH(launch_f32_to_op(h->X, N * d_in, h->op_kind, h->inv_x, h->Xop, h->stream), "X operand");
   }
   if (h->kind == MGFWA_OBJ_NET_OUTPUT &&
@@ -1340,6 +1368,7 @@ mgfwa_status mgfwa_checkpoint_save(mgfwa_t* h, void* host, int64_t bytes) {
   if (!host || bytes != need) return fail(h, MGFWA_EINVAL, "checkpoint: buffer must hold %lld bytes", (long long)need);
   if (h->next_phase != MGFWA_PHASE_EXPLODE) return fail(h, MGFWA_EINVAL, "a debug generation is in progress");
   if (h->cfg.lagged_guiding) return fail(h, MGFWA_EINVAL, "checkpoint: not supported with lagged_guiding");
+  if ((st = ensure_fingerprint(h)) != MGFWA_OK) return st;
   CkptHeader hd{kCkptMagic, h->fingerprint, h->evals, h->launches, h->gen, 0u, ckpt_payload(h)};
   char* out = static_cast<char*>(host) + sizeof(CkptHeader);
   const int64_t F = (int64_t)h->p.B * h->p.mu, B = h->p.B;
@@ -1371,6 +1400,7 @@ mgfwa_status mgfwa_checkpoint_load(mgfwa_t* h, const void* host, int64_t bytes) 
   std::memcpy(&hd, host, sizeof(hd));
   if (hd.magic != kCkptMagic || hd.payload_bytes != ckpt_payload(h))
     return fail(h, MGFWA_EINVAL, "checkpoint: not a checkpoint of this layout");
+  if ((st = ensure_fingerprint(h)) != MGFWA_OK) return st;
   if (hd.fingerprint != h->fingerprint)
     return fail(h, MGFWA_EINVAL, "checkpoint: made for another configuration or objective");
   const char* in = static_cast<const char*>(host) + sizeof(CkptHeader);

@@ -350,6 +350,8 @@ int launch_net_layer(const float* A, int64_t lda, int32_t rows, const float* W, 
 
 // BF16 copy of the first-layer weights of `count` rows (stride ld) into op.
 int launch_to_operand(const float* rows, int64_t ld, int32_t count, const OpDesc& op, cudaStream_t s);
+// *top (0 before) = the bits of the largest magnitude in src[0..n), NaN passed over.
+int launch_abs_max(const float* src, int64_t n, uint32_t* top, cudaStream_t s);
 // dst[e] = BF16(src[e]) or E4M3(src[e] * inv_scale), e < n.
 int launch_f32_to_op(const float* src, int64_t n, int32_t kind, float inv_scale, void* dst, cudaStream_t s);
 
