@@ -1,5 +1,6 @@
-// Fitness kernels on CUDA cores: the FP32 path (GPU-MGFWA, Algorithm 1:
-// "evaluate all the fitness of the sparks"), the fixed-order reduction of
+// Fitness kernels on CUDA cores: the FP32 path of small networks and the
+// FP32 dispatch (GPU-MGFWA, Algorithm 1: "evaluate all the fitness of the
+// sparks"; larger networks: k_fitness_x3.cu), the fixed-order reduction of
 // per-tile partial sums shared with the tensor-core path, the sphere, and
 // the FP64 re-computation of the reported best loss.
 //
