@@ -51,7 +51,7 @@ typedef enum {
 } mgfwa_status;
 
 typedef enum {
-  MGFWA_FP32 = 0, /* FP32 CUDA-core fitness */
+  MGFWA_FP32 = 0, /* FP32 fitness (larger MLPs: first layer on the tensor cores at FP32 accuracy) */
   MGFWA_BF16 = 1, /* tensor cores (tcgen05): BF16 first layer, TF32 later layers, FP32 accumulate; MLPs with
                      d_in % 8 == 0 and two layers (h1 in {32, 64, 128}, <= 32 classes) or three ((h1, h2) in
                      {(128, 64), (64, 32)}, <= 16 classes) */

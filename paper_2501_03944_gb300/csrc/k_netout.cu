@@ -181,7 +181,8 @@ __global__ void __launch_bounds__(256, TR * TC > 32 ? 1 : TR == 4 ? 3 : 2)
 // `ain` the previous layer's FP64 outputs otherwise.  The layer's weights are
 // read once by as many SMs as it has warps; one block reading every row
 // through its own threads, uncoalesced, was one SM's latency-bound chain
-// (1,882 us for the 1000-512x11-1 network, 12 such launches 60 us).
+// (reading back a run of the
+// 1000-512x11-1 network 1,903 us so, 125 us with these 12 launches).
 constexpr int kF64Warps = 4;
 
 __global__ void __launch_bounds__(32 * kF64Warps) k_net_f64_layer(const float* __restrict__ W,
