@@ -30,8 +30,9 @@
 // element, 2 x 4096 elements per 12 MMAs).
 //
 // An operand that is not finite (or rounds to a BF16 infinity) makes every
-// sum it enters non-finite; a sample with such a sum has its sums computed
-// again in FP32 in index order, so infinities and NaN end as they do in k_fitness_simt.
+// sum it enters non-finite; each sum that is not finite, and no other, is
+// computed again in FP32 in index order, so infinities and NaN end as they do
+// in k_fitness_simt and do not reach a neighbour in the tile.
 //
 // Every wait is bounded; a CTA whose wait gives up sets a bit in the status
 // word, writes NaN sums for the tiles it has left and returns.
@@ -214,6 +215,53 @@ __noinline__ __device__ void middle_layer(const Mlp& mlp, const float* P, float*
                                                              act_f(mlp.acts[1], z[u][2]), act_f(mlp.acts[1], z[u][3]));
   }
   epi_bar<kEpiWarps>();
+}
+
+// The activations of the columns c0 + i, i < i_end, whose bit in `mask` is set, of this lane's sample (inputs xr), in
+// FP32 in index order, into h[i * kM].  The warp walks the columns any of its lanes asks for, eight at a time: their W1
+// rows are one broadcast read for all lanes, and their eight chains of FMAs overlap.  Not inlined: rare, and its
+// registers would push out the caller's.
+__noinline__ __device__ void redo_columns(const X3Args& a, const float* xr, int g0, int c0, int i_end, uint64_t mask,
+                                          const float* P, int Tp, float* h) {
+  constexpr int kCols = 8;
+  const int h1 = a.mlp.widths[1], d_in = a.mlp.widths[0];
+  uint64_t any = (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)mask) |
+                 (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(mask >> 32)) << 32;
+  if (i_end < 64) any &= i_end > 0 ? (uint64_t(1) << i_end) - 1 : 0;
+  while (any != 0) {
+    const float* wr[kCols];
+    float z[kCols];
+    int col[kCols], live = 0;
+#pragma unroll
+    for (int u = 0; u < kCols; ++u) {
+      if (any != 0) {
+        col[u] = __ffsll((long long)any) - 1;
+        any &= any - 1;
+        ++live;
+      } else {
+        col[u] = col[0];  // repeated, not stored
+      }
+      const int v = (c0 + col[u]) / h1, r = a.idx ? a.idx[g0 + v] : g0 + v;
+      wr[u] = a.rows + (int64_t)r * a.ld + (int64_t)(c0 + col[u] - v * h1) * d_in;
+      z[u] = 0.0f;
+    }
+    for (int k = 0; k < d_in; k += 4) {
+      const float4 x = __ldg(reinterpret_cast<const float4*>(xr + k));
+#pragma unroll
+      for (int u = 0; u < kCols; ++u) {
+        const float4 w = __ldg(reinterpret_cast<const float4*>(wr[u] + k));
+        z[u] = fmaf(x.x, w.x, z[u]);
+        z[u] = fmaf(x.y, w.y, z[u]);
+        z[u] = fmaf(x.z, w.z, z[u]);
+        z[u] = fmaf(x.w, w.w, z[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kCols; ++u) {
+      const int v = (c0 + col[u]) / h1, j = c0 + col[u] - v * h1;
+      if (u < live && (mask >> col[u] & 1)) h[col[u] * kM] = act_f(a.mlp.acts[0], z[u] + P[v * Tp + j]);
+    }
+  }
 }
 
 // NL: register slots for the logits (C <= NL); kThree: three layers.
@@ -443,20 +491,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
         activate([](float z) { return tanhf(z); });
       else
         activate([](float z) { return fmaxf(z, 0.0f); });
-      const bool bad = !(nan_if_bad == 0.0f);
-      if (bad && n < mlp.N) {
-        // an operand of this sample's sums is not finite: all of them again, in FP32
-        const float* xr = mlp.X + n * d_in;
-        for (int i = 0, j = j0, v = v0; i < kN / 2 && v < V && g0 + v < a.count; ++i) {
-          const float* wr = row_ptr(g0 + v) + (int64_t)j * d_in;
-          float z = 0.0f;
-          for (int k = 0; k < d_in; ++k) z = fmaf(xr[k], wr[k], z);
-          h[i * kM] = act_f(mlp.acts[0], z + P[v * Tp + j]);
-          if (++j == h1) {
-            j = 0;
-            ++v;
-          }
+      // an operand of some sum is not finite: those sums (bit i: column i of this thread's half) again, in FP32
+      const bool bad = n < mlp.N && !(nan_if_bad == 0.0f);
+      if (__any_sync(0xffffffffu, bad)) {
+        uint64_t mask = 0;
+        if (bad) {
+#pragma unroll
+          for (int i = 0; i < kN / 2; ++i)
+            if (!(acc[i] * 0.0f == 0.0f)) mask |= uint64_t(1) << i;
         }
+        const int i_end = min(kN / 2, min(V, a.count - g0) * h1 - half * (kN / 2));  // columns of sparks there are
+        redo_columns(a, mlp.X + (n < mlp.N ? n : mlp.N - 1) * d_in, g0, half * (kN / 2), i_end, mask, P, Tp, h);
       }
       epi_bar<kEpiWarps>();
       const int fl = mlp.widths[L - 1];  // last hidden width
