@@ -60,8 +60,15 @@ constexpr uint32_t kTmemCols = kAcc * kN;
 // mantissas m spread as 1/m, 2^-24 / (2 ln 2).  The epilogue gives it back
 // with the bias, so that the sums' error is as unbiased as a chain of rounded
 // FMAs' (mean relative error of the ReLU networks' losses without it -4.4e-8,
-// with every d_in from 32 to 3072).
-constexpr float kTrunc = 0.7213475f * 0x1p-24f;
+// with every d_in from 32 to 3072).  A sum whose last kExactBits bits are zero
+// is taken as exact and left alone: of numbers that FP32 holds with so many
+// bits to spare (binary or one-hot inputs and coarse weights, say) nothing was
+// lost, and of sums that were rounded one in 2^kExactBits looks so, which the
+// others make up for.  Over 40 drawn networks and batches the geometric mean of
+// the fitness' rms error against 64 bits is 6.6e-8, k_fitness_simt's 9.1e-8.
+constexpr int kExactBits = 4;
+constexpr uint32_t kLastBits = (1u << kExactBits) - 1u;
+constexpr float kTrunc = 0.7213475f * 0x1p-24f * (float)(kLastBits + 1u) / (float)kLastBits;
 
 struct Bars {
   uint64_t full[kMaxStages], empty[kMaxStages];  // a stage's parts are stored; its MMAs have read them
@@ -483,7 +490,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
           for (int i = 0; i < 8; ++i) {
             const float z = acc[i0 + i];
             nan_if_bad = fmaf(z, 0.0f, nan_if_bad);
-            h[(i0 + i) * kM] = act(z + fmaf(z, kTrunc, b1[i]));
+            const float lost = (__float_as_uint(z) & kLastBits) != 0 ? kTrunc : 0.0f;
+            h[(i0 + i) * kM] = act(z + fmaf(z, lost, b1[i]));
           }
         }
       };
