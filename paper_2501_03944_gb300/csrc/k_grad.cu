@@ -517,14 +517,19 @@ int grid_for(int64_t total, int threads = 256) {
 // Output tile width: 64 for narrow products, else 128.
 int tile_n(int64_t Nc) { return Nc <= 64 ? 64 : 128; }
 
+// Output tiles of an M x Nc product.
+int64_t out_tiles(int64_t M, int64_t Nc) {
+  const int bn = tile_n(Nc);
+  return ((M + 127) / 128) * ((Nc + bn - 1) / bn);
+}
+
 // K per split of an M x Nc product with reduction length K: enough splits
 // for two blocks per SM for ONE vector, at least kmin of K each, at most 32.
 // It depends on the product's shape (and the device) only, never on how many
 // vectors share the launch, so a vector's sums -- chunk by chunk, then the
 // chunks in order -- are the same alone or batched.
 int kchunk_for(int64_t M, int64_t Nc, int64_t K, int num_sms, int64_t kmin) {
-  const int bn = tile_n(Nc);
-  const int64_t tiles = ((M + 127) / 128) * ((Nc + bn - 1) / bn);
+  const int64_t tiles = out_tiles(M, Nc);
   int64_t s = (2 * (int64_t)num_sms + tiles - 1) / tiles;
   const int64_t kmax = (K + kmin - 1) / kmin;
   if (s > kmax) s = kmax;
@@ -561,9 +566,13 @@ int gemm_list(const Mlp& mlp, int num_sms, bool forward_only, Gemm* out) {
   if (forward_only) return n;
   for (int l = L - 1; l >= 1; --l) {
     const int64_t fi = mlp.widths[l - 1], fo = mlp.widths[l];
-    // weight gradients: at least 128 samples a chunk (64 wrote and read twice the partials: with 8 vectors of the
-    // 784-64-10 network 32 chunks 224 us a call, 16 chunks 214; with one 107 either way)
-    out[n++] = shape(fi + 1, fo, N, num_sms, 128);
+    // weight gradients: at least 128 samples a chunk, where the tiles times such chunks occupy most SMs with one vector
+    // (64 samples a chunk write and read twice the partials: 8 vectors of 784-64-10, N = 2048, 224 us a call with 64,
+    // 214 with 128; 784-128-10 325 and 304), else 64, whose blocks are twice as many and half as long (16-64-10, N =
+    // 512, one vector 57 us with 64, 65 with 128; 120-64-10, N = 2048, two vectors 78 and 82).  Over d_in 16 to 1024, N
+    // 100 to 4096 and 1 to 16 vectors the two are within 2% of each other from a quarter of the SMs up to here.
+    const bool fills = 3 * out_tiles(fi + 1, fo) * ((N + 127) / 128) >= 2 * (int64_t)num_sms;
+    out[n++] = shape(fi + 1, fo, N, num_sms, fills ? 128 : 64);
     if (l > 1) out[n++] = shape(N, fi, fo, num_sms);
   }
   return n;
