@@ -55,7 +55,7 @@ __global__ void k_rank(Problem p, float* __restrict__ fit_e, int32_t* __restrict
   }
 }
 
-constexpr int kSelThreads = 256;
+constexpr int kSelThreads = 32 * kSelWarps;
 constexpr int kSelStage = 1024;  // fireworks per run whose fitness the selection's serial part reads from shared memory
 constexpr int kSelChunk = 8;     // candidates per lane loaded before they are compared
 constexpr int kPickStage = 2048; // candidates per firework the elite pick stages in shared memory

@@ -262,9 +262,16 @@ bool rescore_on(const mgfwa_t* h) {
 bool finish_in_rank(const mgfwa_t* h) { return h->capturing && h->kind == MGFWA_OBJ_MLP_CE; }
 bool finish_in_pick(const mgfwa_t* h) { return h->capturing && rescore_on(h); }
 // (not with lagged guiding, whose one launch's sums are finished before the rank, nor for a member of a grouped
-// fitness launch, whose capture skips the guiding evaluation and finishes its sums itself)
+// fitness launch, whose capture skips the guiding evaluation and finishes its sums itself).  The selection has one
+// block of kSelWarps warps per run: a warp takes its fireworks in turn, their guiding sparks 32 at a time and a
+// spark's sample tiles eight at a time, each step a round trip to L2, where a launch of its own spreads all sums over
+// the GPU.  Measured (8-16-3, us a generation, finished here / by its own launch): one such step 21.0 / 23.0 (5
+// fireworks, 4 guiding sparks, N = 512), two 25.3 / 27.1 (the same, N = 2048) and 23.1 / 23.0 (16, 1, 512), three 35.4 /
+// 35.3, four 41.3 / 40.6, sixteen 89.8 / 76.5 (128, 4, 512), 128 542 / 442 (1,024, 4, 512); so up to two.
 bool finish_in_select(const mgfwa_t* h) {
-  return h->capturing && !h->grouped_fit && h->kind == MGFWA_OBJ_MLP_CE && !rescore_on(h) && !h->lag_now;
+  const Problem& p = h->p;
+  const int64_t steps = (int64_t)((p.mu + kSelWarps - 1) / kSelWarps) * ((p.m + 31) / 32) * ((h->mtiles + 7) / 8);
+  return h->capturing && !h->grouped_fit && h->kind == MGFWA_OBJ_MLP_CE && !rescore_on(h) && !h->lag_now && steps <= 2;
 }
 
 // Generation `gen` (1-based) ends with a hybrid refinement.

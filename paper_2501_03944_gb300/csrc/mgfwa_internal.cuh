@@ -285,6 +285,9 @@ int launch_guide(const Problem& p, const uint32_t* gens_done, const float* fw_x,
 int launch_run_best_init(const Problem& p, const float* fw_x, const float* fw_f, float* best_x, float* best_f,
                          cudaStream_t s);
 
+// Warps of the selection's block (one block per run).
+constexpr int kSelWarps = 8;
+
 // Selection of every firework (winner[z]: its winning candidate or -1) and
 // each run's best-so-far (winner[B*mu + b]: the run's improving firework or
 // -1; winner[B*mu + B]: the generation; winner holds B*mu + B + 1
