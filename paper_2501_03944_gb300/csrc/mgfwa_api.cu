@@ -490,8 +490,9 @@ int32_t overlap_tiles(const mgfwa_t* h) {
 // `side` while the pair kernel evaluates chunk c on the handle's stream.  The
 // sampler is bound by integer arithmetic and writes, the pair kernel by the
 // tensor cores, and the pair kernel's one CTA per SM leaves registers for a
-// few sampler blocks beside it; its launches have the higher priority, so that
-// its CTAs are placed first.
+// few sampler blocks beside it; its launches have a priority one step above the
+// sampler's (the default), so that its CTAs are placed first and no stream that
+// asked for more than that is outranked.
 mgfwa_status explode_eval_overlapped(mgfwa_t* h, int32_t per, cudaStream_t side, std::vector<cudaEvent_t>& ev) {
   const Problem& p = h->p;
   const int64_t n_e = (int64_t)p.B * p.mu * p.lam;
@@ -499,7 +500,7 @@ mgfwa_status explode_eval_overlapped(mgfwa_t* h, int32_t per, cudaStream_t side,
   int least = 0, greatest = 0;
   if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess) return cuda_fail(h, "stream priorities");
   TcPlan tc = h->tc;
-  tc.priority = greatest;
+  tc.priority = greatest < least ? least - 1 : 0;  // numerically lower is higher
   tc.partial_stride = n_e;
   const int64_t chunk = (int64_t)per * h->tc.sparks_per_tile;
   for (int64_t r0 = 0; r0 < n_e; r0 += chunk) {
