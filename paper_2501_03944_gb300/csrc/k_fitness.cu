@@ -428,8 +428,12 @@ int launch_fitness_fp32(const Mlp& mlp, const float* rows, int64_t ld, int32_t c
   if (count <= 0) return 0;
   const int mtiles = (int)((mlp.N + kMT - 1) / kMT);
   if (small_net(mlp, 8, 16, 3)) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return -1;
     // one spark per block while one block per SM slot (16 of 128 threads) holds them, then up to kSmallSparks
-    const int64_t pairs = (int64_t)count * mtiles, slots = 152 * 16;
+    const int64_t pairs = (int64_t)count * mtiles, slots = (int64_t)sms * 16;
     const int per = (int)(pairs <= slots ? 1 : (pairs / slots < kSmallSparks ? pairs / slots : kSmallSparks));
     dim3 grid((count + per - 1) / per, mtiles);
     return launch_pdl(k_fitness_small<8, 16, 3>, grid, dim3(kMT), 0, s, mlp, rows, ld, count, (int32_t)per, idx,
