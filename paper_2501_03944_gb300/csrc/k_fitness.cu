@@ -28,13 +28,12 @@ __host__ __device__ __forceinline__ int odd_ld(int w) { return w + ((w & 1) == 0
 // tile stays in shared memory, later layers run one sample per thread, and
 // the block's cross-entropy sum goes to partial[mt][row].
 __global__ void __launch_bounds__(kThreads) k_fitness_simt(Mlp mlp, const float* __restrict__ rows, int64_t ld,
-                                                           int32_t count, const int32_t* __restrict__ idx,
-                                                           float* __restrict__ partial) {
+                                                           int32_t count, float* __restrict__ partial) {
   griddep_wait();
   griddep_launch_dependents();
   extern __shared__ __align__(16) float smem[];
   const int row = blockIdx.x, mt = blockIdx.y;
-  const float* w = rows + (int64_t)(idx != nullptr ? idx[row] : row) * ld;
+  const float* w = rows + (int64_t)row * ld;
   const int L = mlp.n_layers;
   const int d_in = mlp.widths[0], h1 = mlp.widths[1];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -198,8 +197,7 @@ constexpr int kSmallSparks = 8;
 
 template <int DI, int H1, int C>
 __global__ void __launch_bounds__(kMT) k_fitness_small(Mlp mlp, const float* __restrict__ rows, int64_t ld,
-                                                       int32_t count, int32_t per, const int32_t* __restrict__ idx,
-                                                       float* __restrict__ partial) {
+                                                       int32_t count, int32_t per, float* __restrict__ partial) {
   using Net = SmallNet<DI, H1, C>;
   __shared__ float ws[kSmallSparks][Net::D];
   __shared__ float red[kSmallSparks][kMT / 32];
@@ -209,8 +207,7 @@ __global__ void __launch_bounds__(kMT) k_fitness_small(Mlp mlp, const float* __r
   const int gs = min(per, count - s0);
   for (int e = threadIdx.x; e < gs * Net::D; e += kMT) {
     const int g = e / Net::D, k = e - g * Net::D;
-    const int r = s0 + g;
-    ws[g][k] = rows[(int64_t)(idx != nullptr ? idx[r] : r) * ld + k];
+    ws[g][k] = rows[(int64_t)(s0 + g) * ld + k];
   }
   const int64_t n = (int64_t)mt * kMT + threadIdx.x;
   const bool valid = n < mlp.N;
@@ -244,12 +241,12 @@ bool small_net(const Mlp& mlp, int di, int h1, int c) {
 }
 
 __global__ void k_fitness_finish(const float* __restrict__ partial, int32_t mtiles, int32_t count, float n_f,
-                                 const int32_t* __restrict__ idx, float* __restrict__ fit) {
+                                 float* __restrict__ fit) {
   griddep_wait();
   griddep_launch_dependents();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= count) return;
-  fit[idx != nullptr ? idx[r] : r] = __fdiv_rn(tile_sum(partial, r, count, mtiles), n_f);
+  fit[r] = __fdiv_rn(tile_sum(partial, r, count, mtiles), n_f);
 }
 
 __global__ void __launch_bounds__(256) k_sphere(const float* __restrict__ rows, int64_t ld, int64_t D,
@@ -412,19 +409,16 @@ size_t smem_for(const Mlp& mlp) {
 
 }  // namespace
 
-size_t fitness_simt_smem_bytes(const Mlp& mlp) { return smem_for(mlp); }
-
-int launch_fitness_finish(const float* partial, int32_t mtiles, int32_t count, int64_t N, float* fit,
-                          cudaStream_t s, const int32_t* idx) {
+int launch_fitness_finish(const float* partial, int32_t mtiles, int32_t count, int64_t N, float* fit, cudaStream_t s) {
   if (count <= 0) return 0;
   return launch_pdl(k_fitness_finish, dim3((count + 255) / 256), dim3(256), 0, s, partial, mtiles, count, (float)N,
-                    idx, fit) == cudaSuccess
+                    fit) == cudaSuccess
              ? 1
              : -1;
 }
 
 int launch_fitness_fp32(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial,
-                        uint32_t* status, cudaStream_t s, const int32_t* idx) {
+                        uint32_t* status, cudaStream_t s) {
   if (count <= 0) return 0;
   const int mtiles = (int)((mlp.N + kMT - 1) / kMT);
   if (small_net(mlp, 8, 16, 3)) {
@@ -436,16 +430,16 @@ int launch_fitness_fp32(const Mlp& mlp, const float* rows, int64_t ld, int32_t c
     const int64_t pairs = (int64_t)count * mtiles, slots = (int64_t)sms * 16;
     const int per = (int)(pairs <= slots ? 1 : (pairs / slots < kSmallSparks ? pairs / slots : kSmallSparks));
     dim3 grid((count + per - 1) / per, mtiles);
-    return launch_pdl(k_fitness_small<8, 16, 3>, grid, dim3(kMT), 0, s, mlp, rows, ld, count, (int32_t)per, idx,
-                      partial) == cudaSuccess
+    return launch_pdl(k_fitness_small<8, 16, 3>, grid, dim3(kMT), 0, s, mlp, rows, ld, count, (int32_t)per, partial) ==
+                   cudaSuccess
                ? 1
                : -1;
   }
-  if (fitness_x3_ok(mlp)) return launch_fitness_x3(mlp, rows, ld, count, partial, status, s, idx);
+  if (fitness_x3_ok(mlp)) return launch_fitness_x3(mlp, rows, ld, count, partial, status, s);
   const size_t smem = smem_for(mlp);
   if (ensure_smem_limit<k_fitness_simt>(smem) != cudaSuccess) return -1;
   dim3 grid(count, mtiles);
-  return launch_pdl(k_fitness_simt, grid, dim3(kThreads), smem, s, mlp, rows, ld, count, idx, partial) == cudaSuccess
+  return launch_pdl(k_fitness_simt, grid, dim3(kThreads), smem, s, mlp, rows, ld, count, partial) == cudaSuccess
              ? 1
              : -1;
 }

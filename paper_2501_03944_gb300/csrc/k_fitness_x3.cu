@@ -83,7 +83,6 @@ struct X3Args {
   Mlp mlp;
   const float* rows;
   int64_t ld;
-  const int32_t* idx;
   int32_t count, mtiles, tiles;  // tiles = mtiles * ceil(count / V), sample tile fastest
   int32_t V, stages;
   float* partial;                // [mtiles][count]
@@ -269,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
   griddep_wait();
   griddep_launch_dependents();
 
-  auto row_ptr = [&](int spark) { return a.rows + (int64_t)(a.idx ? a.idx[spark] : spark) * a.ld; };
+  auto row_ptr = [&](int spark) { return a.rows + (int64_t)spark * a.ld; };
 
   if (warp < kConvWarps) {
     // ---- load and split: this thread takes inputs 4 c .. 4 c + 3 of a block (a row's 32 inputs are one 128-byte
@@ -579,7 +578,7 @@ bool fitness_x3_ok(const Mlp& mlp) {
 }
 
 int launch_fitness_x3(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial, uint32_t* status,
-                      cudaStream_t s, const int32_t* idx) {
+                      cudaStream_t s) {
   if (count <= 0) return 0;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -589,7 +588,6 @@ int launch_fitness_x3(const Mlp& mlp, const float* rows, int64_t ld, int32_t cou
   a.mlp = mlp;
   a.rows = rows;
   a.ld = ld;
-  a.idx = idx;
   a.count = count;
   a.V = sparks_per_tile(mlp);
   // few sparks: fewer to a tile, so that the tiles reach more SMs

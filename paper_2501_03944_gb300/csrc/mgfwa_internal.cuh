@@ -303,23 +303,21 @@ int launch_select(const Problem& p, const float* fit_e, float* fit_g, const floa
                   float* best_x, float* best_f, uint32_t* gens_done, float* f_old, int32_t* loser, cudaStream_t s,
                   const float* partial = nullptr, int32_t mtiles = 0, int64_t N = 0);
 
-// FP32 fitness of `count` rows (stride `ld` floats; row r is rows[idx[r]]
-// when idx is given): per-(m-tile, r) partial cross-entropy sums into
-// `partial` [mtiles][count] (the mean is taken by launch_fitness_finish).
+// FP32 fitness of `count` rows (stride `ld` floats): per-(m-tile, r) partial
+// cross-entropy sums into `partial` [mtiles][count] (the mean is taken by
+// launch_fitness_finish).
 // With fitness_x3_ok the first layer runs on the tensor cores at FP32
 // accuracy (k_fitness_x3.cu; a device wait that gives up sets *status and
 // leaves NaN), else everything on the CUDA cores.
 int launch_fitness_fp32(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial,
-                        uint32_t* status, cudaStream_t s, const int32_t* idx = nullptr);
+                        uint32_t* status, cudaStream_t s);
 bool fitness_x3_ok(const Mlp& mlp);
 int launch_fitness_x3(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial, uint32_t* status,
-                      cudaStream_t s, const int32_t* idx = nullptr);
-size_t fitness_simt_smem_bytes(const Mlp& mlp);
+                      cudaStream_t s);
 
-// fit[r] (fit[idx[r]] when idx is given) = mean over m-tiles of partial:
+// fit[r] = mean over m-tiles of partial:
 // fixed-order FP32 sum / N.
-int launch_fitness_finish(const float* partial, int32_t mtiles, int32_t count, int64_t N, float* fit,
-                          cudaStream_t s, const int32_t* idx = nullptr);
+int launch_fitness_finish(const float* partial, int32_t mtiles, int32_t count, int64_t N, float* fit, cudaStream_t s);
 
 // Elite candidates for the FP32 re-score: per firework (all runs) the
 // `E` best of its lam explosion and m guiding sparks by the current
