@@ -87,7 +87,8 @@ MGFWA_API mgfwa_status mgfwa_debug_fp32_tc(const mgfwa_t* h, int32_t* rescore, i
 MGFWA_API mgfwa_status mgfwa_debug_profile(mgfwa_t* h, int32_t enable);
 MGFWA_API mgfwa_status mgfwa_debug_kernel_times(mgfwa_t* h, double* ms_out, int64_t* launches_out);
 /* Budget, in SM clock ticks (clock64), of every bounded mbarrier wait in the
- * handle's tensor-core fitness kernels, for launches made after the call
+ * handle's tensor-core fitness kernels (BF16, E4M3, the first layer of FP32,
+ * the layers of FP32X3), for launches made after the call
  * (0 restores the default of about 2 s; a generation graph captured earlier
  * keeps the budget it was captured with).  With a budget of a few ticks an
  * ordinary wait runs out: the kernel raises its abort flag, every role leaves

@@ -65,6 +65,7 @@ struct NetX3Plan {
   uint32_t* w_parts[kNetMaxLayers] = {};
   float* partial = nullptr;  // the split layers' partial sums [splits][max_rows][fan_out]
   int64_t max_rows = 0;
+  uint64_t wait_budget = 0;  // clock64 ticks before a bounded wait gives up (0 = the default, ~2 s)
 };
 bool net_x3_layer(int fan_in, int fan_out);
 // 32-bit words of the plan's buffers (two BF16 per word).

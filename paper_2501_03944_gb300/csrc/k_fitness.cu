@@ -418,7 +418,7 @@ int launch_fitness_finish(const float* partial, int32_t mtiles, int32_t count, i
 }
 
 int launch_fitness_fp32(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial,
-                        uint32_t* status, cudaStream_t s) {
+                        uint32_t* status, uint64_t wait_budget, cudaStream_t s) {
   if (count <= 0) return 0;
   const int mtiles = (int)((mlp.N + kMT - 1) / kMT);
   if (small_net(mlp, 8, 16, 3)) {
@@ -435,7 +435,7 @@ int launch_fitness_fp32(const Mlp& mlp, const float* rows, int64_t ld, int32_t c
                ? 1
                : -1;
   }
-  if (fitness_x3_ok(mlp)) return launch_fitness_x3(mlp, rows, ld, count, partial, status, s);
+  if (fitness_x3_ok(mlp)) return launch_fitness_x3(mlp, rows, ld, count, partial, status, wait_budget, s);
   const size_t smem = smem_for(mlp);
   if (ensure_smem_limit<k_fitness_simt>(smem) != cudaSuccess) return -1;
   dim3 grid(count, mtiles);

@@ -35,7 +35,7 @@
 // in k_fitness_simt and do not reach a neighbour in the tile.
 //
 // Every wait is bounded; a CTA whose wait gives up sets a bit in the status
-// word, writes NaN sums for the tiles it has left and returns.
+// word, if there is one, writes NaN sums for the tiles it has left and returns.
 #include "mgfwa_internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -76,6 +76,7 @@ struct Bars {
   uint64_t done;
   uint32_t tmem_base;
   volatile int abort_flag;
+  uint64_t wait_budget;   // clock64 ticks before a wait gives up
   float red[kMaxV][kM / 32];
 };
 
@@ -86,7 +87,8 @@ struct X3Args {
   int32_t count, mtiles, tiles;  // tiles = mtiles * ceil(count / V), sample tile fastest
   int32_t V, stages;
   float* partial;                // [mtiles][count]
-  uint32_t* status;
+  uint32_t* status;              // null: not reported
+  uint64_t wait_budget;          // clock64 ticks before a wait gives up
 };
 
 __device__ __forceinline__ float act_f(int a, float v) { return a == kActTanh ? tanhf(v) : fmaxf(v, 0.0f); }
@@ -101,10 +103,33 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
   return d;
 }
 
-// A whole warp's bounded wait: every lane leaves with the same answer.
-__device__ __forceinline__ bool warp_wait(volatile int* abort, uint64_t* bar, uint32_t parity, uint32_t* status,
-                                          uint32_t code) {
-  return __all_sync(0xffffffffu, mbar_wait(abort, bar, parity, status, code));
+// A bounded wait (its limit read from shared memory, and only while it waits, so that it holds no registers).
+__device__ __forceinline__ bool wait(Bars* sb, uint64_t* bar, uint32_t parity, uint32_t* status, uint32_t code) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, parity)) {
+    if (sb->abort_flag) return false;
+    if ((uint64_t)(clock64() - t0) > sb->wait_budget) {
+      sb->abort_flag = 1;
+      if (status != nullptr) atomicOr(status, code);
+      return false;
+    }
+  }
+  return true;
+}
+// The wait for every issued MMA before the CTA leaves (ignores the abort flag).
+__device__ __forceinline__ void drain(uint64_t* bar, uint32_t* status) {
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, 0u)) {
+    if ((uint64_t)(clock64() - t0) > kWaitBudget) {
+      if (status != nullptr) atomicOr(status, 16u);
+      return;
+    }
+  }
+}
+// A whole warp's wait: every lane leaves with the same answer.
+__device__ __forceinline__ bool warp_wait(Bars* sb, uint64_t* bar, uint32_t parity, uint32_t* status, uint32_t code) {
+  return __all_sync(0xffffffffu, wait(sb, bar, parity, status, code));
 }
 
 // Four consecutive inputs -> their three BF16 parts, 8 bytes each.
@@ -251,6 +276,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
     }
     mbar_init(&sb->done, 1);
     sb->abort_flag = 0;
+    sb->wait_budget = a.wait_budget;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -264,7 +290,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sb->tmem_base;
-  volatile int* abort = &sb->abort_flag;
   griddep_wait();
   griddep_launch_dependents();
 
@@ -301,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
 #pragma unroll
       for (int i = 0; i < kTasks; ++i) load(i, 0);
       for (int kb = 0; kb < nkb; ++kb) {
-        if (!warp_wait(abort, &sb->empty[s], ph, a.status, 1u)) {
+        if (!warp_wait(sb, &sb->empty[s], ph, a.status, 1u)) {
           dead = true;
           break;
         }
@@ -336,8 +361,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
       bool dead = false;
       for (int t = blockIdx.x; t < a.tiles && !dead; t += gridDim.x) {
         for (int kb = 0; kb < nkb; ++kb) {
-          if (!mbar_wait(abort, &sb->full[s], ph, a.status, 2u) ||
-              !mbar_wait(abort, &sb->acc_empty[b], aph, a.status, 4u)) {
+          if (!wait(sb, &sb->full[s], ph, a.status, 2u) ||
+              !wait(sb, &sb->acc_empty[b], aph, a.status, 4u)) {
             dead = true;
             break;
           }
@@ -371,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
         }
       }
       mma_commit(&sb->done);  // after every issued MMA
-      mbar_drain(&sb->done, 0u, a.status);
+      drain(&sb->done, a.status);
     }
   } else {
     const int ew = warp - kConvWarps, q = warp & 3, half = ew >> 2;
@@ -399,7 +424,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
       for (int i = 0; i < kN / 2; ++i) acc[i] = 0.0f;
       bool dead = false;
       for (int kb = 0; kb < nkb; ++kb) {
-        if (!warp_wait(abort, &sb->acc_full[b], ph, a.status, 8u)) {
+        if (!warp_wait(sb, &sb->acc_full[b], ph, a.status, 8u)) {
           dead = true;
           break;
         }
@@ -578,7 +603,7 @@ bool fitness_x3_ok(const Mlp& mlp) {
 }
 
 int launch_fitness_x3(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial, uint32_t* status,
-                      cudaStream_t s) {
+                      uint64_t wait_budget, cudaStream_t s) {
   if (count <= 0) return 0;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -601,6 +626,8 @@ int launch_fitness_x3(const Mlp& mlp, const float* rows, int64_t ld, int32_t cou
   a.stages = smem_for(mlp, a.V, kMaxStages) <= kSmemLimit ? kMaxStages : kMaxStages - 1;
   a.partial = partial;
   a.status = status;
+  // a tile whose sums all end in infinities is 64 chains of d_in steps, each a read from L2, while the other warps wait
+  a.wait_budget = wait_budget != 0 ? wait_budget : kWaitBudget + ((uint64_t)mlp.widths[0] << 15);
   const size_t smem = smem_for(mlp, a.V, a.stages);
   const dim3 grid((unsigned)(tiles < sms ? tiles : sms));
   cudaError_t e;

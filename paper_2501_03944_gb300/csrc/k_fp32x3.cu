@@ -76,12 +76,13 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
   return ok != 0;
 }
 // Bounded wait; false once this CTA aborts.
-__device__ __forceinline__ bool mbar_wait(Bars* sb, uint64_t* b, uint32_t parity, uint32_t* status, uint32_t code) {
+__device__ __forceinline__ bool mbar_wait(Bars* sb, uint64_t* b, uint32_t parity, uint32_t* status, uint32_t code,
+                                          uint64_t budget = kWaitBudget) {
   if (mbar_try(b, parity)) return true;
   const long long t0 = clock64();
   while (!mbar_try(b, parity)) {
     if (sb->abort_flag) return false;
-    if ((uint64_t)(clock64() - t0) > kWaitBudget) {
+    if ((uint64_t)(clock64() - t0) > budget) {
       sb->abort_flag = 1;
       atomicOr(status, code);
       return false;
@@ -668,6 +669,7 @@ struct NetX3Args {
   uint32_t* parts;     // the output's BF16 parts, plane p at parts + p * plane_words, row r at + r * n / 2; or null
   int64_t plane_words;
   uint32_t* status;
+  uint64_t wait_budget;  // clock64 ticks before a wait gives up
 };
 
 __device__ __forceinline__ float net_act(int a, float v) {
@@ -805,7 +807,7 @@ __global__ void __launch_bounds__(kNetThreads, 1)
       for (int kb = 0; kb < first; ++kb) load_a(kb);
       int kb = first;
       for (; kb < nkb; ++kb) {
-        if (!mbar_wait(sb, &sb->empty[kb % S], (uint32_t)(kb / S - 1) & 1u, a.status, 1u)) break;
+        if (!mbar_wait(sb, &sb->empty[kb % S], (uint32_t)(kb / S - 1) & 1u, a.status, 1u, a.wait_budget)) break;
         mbar_expect_tx(&sb->full[kb % S], kStageBytes);
         load_w(kb);
         load_a(kb);
@@ -820,11 +822,11 @@ __global__ void __launch_bounds__(kNetThreads, 1)
       bool ok = true;
       for (int i = 0; i < nsp; ++i) {
         // the accumulators are free once the epilogue has read the split before
-        if (ok && i > 0) ok = mbar_wait(sb, &sb->read, (uint32_t)(i - 1) & 1u, a.status, 4u);
+        if (ok && i > 0) ok = mbar_wait(sb, &sb->read, (uint32_t)(i - 1) & 1u, a.status, 4u, a.wait_budget);
         const int k1 = min((i + 1) * kNetKPer, nkb);
         for (int kb = i * kNetKPer; ok && kb < k1; ++kb) {
           const int s = kb % S, l = kb - i * kNetKPer;  // l: block of the split
-          if (!mbar_wait(sb, &sb->full[s], (uint32_t)(kb / S) & 1u, a.status, 2u)) {
+          if (!mbar_wait(sb, &sb->full[s], (uint32_t)(kb / S) & 1u, a.status, 2u, a.wait_budget)) {
             ok = false;
             break;
           }
@@ -1116,6 +1118,7 @@ int launch_net_output_x3(const NetX3Plan& pl, const NetOut& net, const float* ro
       x.parts = next_tc ? pl.act_parts[(l + 1) & 1] : nullptr;
       x.plane_words = pl.max_rows * (fo / 2);
       x.status = status;
+      x.wait_budget = pl.wait_budget != 0 ? pl.wait_budget : kWaitBudget;
       const dim3 grid((unsigned)((count + kBM - 1) / kBM), (unsigned)((fo + kN - 1) / kN),
                       (unsigned)((x.splits + x.per - 1) / x.per));
       if (launch_pdl_z(k_net_x3, grid, dim3(kNetThreads), net_x3_smem(x.per), x.partial ? 1u : grid.z, s,

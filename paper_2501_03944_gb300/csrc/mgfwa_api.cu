@@ -241,7 +241,9 @@ mgfwa_status eval_rows(mgfwa_t* h, int64_t first, int32_t count, int32_t precisi
                                      h->status, h->stream),
                 "tensor-core fitness");
     else
-      MG_LAUNCH(h, launch_fitness_fp32(h->mlp, rows, h->p.Dp, count, h->partial, h->status, h->stream), "FP32 fitness");
+      MG_LAUNCH(h, launch_fitness_fp32(h->mlp, rows, h->p.Dp, count, h->partial, h->status, h->tc.wait_budget,
+                                       h->stream),
+                "FP32 fitness");
   }
   if (defer_finish) return MGFWA_OK;
   Mark mk(h, G_FINISH);
@@ -1915,6 +1917,7 @@ mgfwa_status mgfwa_debug_fp32_tc(const mgfwa_t* h, int32_t* rescore, int32_t* re
 mgfwa_status mgfwa_debug_wait_budget(mgfwa_t* h, uint64_t ticks) {
   if (!h) return MGFWA_EINVAL;
   h->tc.wait_budget = ticks;
+  h->net_x3.wait_budget = ticks;
   return MGFWA_OK;
 }
 

@@ -307,13 +307,14 @@ int launch_select(const Problem& p, const float* fit_e, float* fit_g, const floa
 // cross-entropy sums into `partial` [mtiles][count] (the mean is taken by
 // launch_fitness_finish).
 // With fitness_x3_ok the first layer runs on the tensor cores at FP32
-// accuracy (k_fitness_x3.cu; a device wait that gives up sets *status and
-// leaves NaN), else everything on the CUDA cores.
+// accuracy (k_fitness_x3.cu; a device wait that gives up, after wait_budget
+// clock64 ticks or, 0, the default, sets *status where one is given and leaves
+// NaN), else everything on the CUDA cores.
 int launch_fitness_fp32(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial,
-                        uint32_t* status, cudaStream_t s);
+                        uint32_t* status, uint64_t wait_budget, cudaStream_t s);
 bool fitness_x3_ok(const Mlp& mlp);
 int launch_fitness_x3(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial, uint32_t* status,
-                      cudaStream_t s);
+                      uint64_t wait_budget, cudaStream_t s);
 
 // fit[r] = mean over m-tiles of partial:
 // fixed-order FP32 sum / N.

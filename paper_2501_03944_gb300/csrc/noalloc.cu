@@ -31,19 +31,15 @@ namespace {
 // Partial sums, [sample tiles of 128][count]; every entry a call reads is
 // written by the same call first, so nothing needs clearing between calls.
 constexpr int64_t kScratchFloats = int64_t(1) << 18;
-struct Scratch {
-  float partial[kScratchFloats];
-  uint32_t status;  // where a device wait that gives up leaves its code (the fitness is NaN then)
-};
-__device__ __align__(256) Scratch g_noalloc;
+__device__ __align__(256) float g_noalloc_partial[kScratchFloats];
 
 constexpr int kMaxDevices = 64;
-Scratch* g_scratch[kMaxDevices] = {};
+float* g_scratch[kMaxDevices] = {};
 std::mutex g_scratch_mu;
 
 // Device address of the scratch array on the current device (looked up on
 // the first call that runs on that device).
-cudaError_t scratch_on_current_device(Scratch** out) {
+cudaError_t scratch_on_current_device(float** out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -51,9 +47,9 @@ cudaError_t scratch_on_current_device(Scratch** out) {
   std::lock_guard<std::mutex> lock(g_scratch_mu);
   if (g_scratch[dev] == nullptr) {
     void* p = nullptr;
-    e = cudaGetSymbolAddress(&p, g_noalloc);
+    e = cudaGetSymbolAddress(&p, g_noalloc_partial);
     if (e != cudaSuccess) return e;
-    g_scratch[dev] = static_cast<Scratch*>(p);
+    g_scratch[dev] = static_cast<float*>(p);
   }
   *out = g_scratch[dev];
   return cudaSuccess;
@@ -118,14 +114,15 @@ extern "C" MGFWA_API mgfwa_status mgfwa_evaluate_fp32_noalloc(int32_t n_layers, 
   mlp.y = y_dev;
   mlp.w1_elems = (int64_t)widths[0] * widths[1];
 
-  Scratch* scratch = nullptr;
+  float* scratch = nullptr;
   if (scratch_on_current_device(&scratch) != cudaSuccess) {
     cudaGetLastError();
     return reject(MGFWA_ECUDA, "noalloc: cudaGetSymbolAddress of the scratch array failed");
   }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  if (mgfwa::launch_fitness_fp32(mlp, rows_dev, ld, count, scratch->partial, &scratch->status, s) < 0 ||
-      mgfwa::launch_fitness_finish(scratch->partial, (int32_t)mtiles, count, n_samples, fitness_dev, s) < 0) {
+  // no status word: a device wait that gives up shows as NaN fitness
+  if (mgfwa::launch_fitness_fp32(mlp, rows_dev, ld, count, scratch, nullptr, 0, s) < 0 ||
+      mgfwa::launch_fitness_finish(scratch, (int32_t)mtiles, count, n_samples, fitness_dev, s) < 0) {
     cudaError_t e = cudaGetLastError();
     char msg[160];
     snprintf(msg, sizeof(msg), "noalloc: kernel launch failed: %s", cudaGetErrorString(e));
