@@ -240,7 +240,9 @@ MGFWA_API mgfwa_status mgfwa_get_info(const mgfwa_t* h, mgfwa_info* info);
  * may differ) and objective (a fingerprint of both is checked: EINVAL
  * otherwise), between
  * generations, and the run then continues exactly as the saved one would
- * have.  Both calls synchronise. */
+ * have.  Both calls synchronise.  The fingerprint is taken at a handle's first
+ * save or load, not at create: a strided read of the batch back to the host
+ * (0.15 ms more than a later save for 2048 x 784, 1 ms for 4096 x 3072). */
 MGFWA_API mgfwa_status mgfwa_checkpoint_size(const mgfwa_t* h, int64_t* bytes);
 MGFWA_API mgfwa_status mgfwa_checkpoint_save(mgfwa_t* h, void* host, int64_t bytes);
 MGFWA_API mgfwa_status mgfwa_checkpoint_load(mgfwa_t* h, const void* host, int64_t bytes);
