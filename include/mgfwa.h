@@ -51,8 +51,9 @@ typedef enum {
 } mgfwa_status;
 
 typedef enum {
-  MGFWA_FP32 = 0, /* FP32 fitness.  MLPs with d_in >= 16, h1 in 8..128 (three layers: h2 <= 64) and
-                     d_in h1 n_samples >= 2^20 take the first layer to the tensor cores at FP32 accuracy: operands as
+  MGFWA_FP32 = 0, /* FP32 fitness.  MLPs with d_in >= 16, h1 in 8..128 (three layers: h2 <= 64),
+                     d_in h1 n_samples >= 2^20 and later layers that do not outweigh the first take the first layer to
+                     the tensor cores at FP32 accuracy: operands as
                      three BF16 parts, six products, sums of 32 inputs truncated to FP32, those added rounded to
                      nearest and the mean truncation given back, sums of whole numbers (times a power of two) of up to
                      20 bits exact (rms error of the fitness against 64 bits 6.3e-8, with FP32 FMAs in index order

@@ -409,6 +409,19 @@ size_t smem_for(const Mlp& mlp) {
 
 }  // namespace
 
+// What k_fitness_simt takes for 128 samples of a spark, as a share of an SM
+// (fitted, as tile_ns in k_fitness_x3.cu): the first layer in steps of 16
+// inputs and 64 hidden units, the later ones a sample a thread.  Where the
+// activations leave room for one block per SM only it is a third slower.
+int64_t fitness_simt_ns(const Mlp& mlp) {
+  const int L = mlp.n_layers, h1 = mlp.widths[1], h2 = L == 3 ? mlp.widths[2] : 0;
+  const int64_t pairs = (int64_t)(h2 + 1) / 2 * h1 + (int64_t)(mlp.widths[L] + 1) / 2 * mlp.widths[L - 1];
+  const int64_t ns = 69LL * ((mlp.widths[0] + kKT - 1) / kKT * kKT) * ((h1 + kHC - 1) / kHC) + 18 * h1 + 11 * pairs +
+                     (mlp.acts[0] == kActTanh ? 9 * h1 : 0) + (L == 3 && mlp.acts[1] == kActTanh ? 9 * h2 : 0);
+  const size_t blocks = 232448 / (smem_for(mlp) + 1024);  // 227 KB per SM, 1 KB of each block's reserved
+  return blocks < 2 ? ns * 4 / 3 : blocks > 2 ? ns * 9 / 10 : ns;
+}
+
 int launch_fitness_finish(const float* partial, int32_t mtiles, int32_t count, int64_t N, float* fit, cudaStream_t s) {
   if (count <= 0) return 0;
   return launch_pdl(k_fitness_finish, dim3((count + 255) / 256), dim3(256), 0, s, partial, mtiles, count, (float)N,

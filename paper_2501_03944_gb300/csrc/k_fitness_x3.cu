@@ -591,15 +591,44 @@ constexpr size_t kSmemLimit = 232448;  // 227 KB per block
 // spark's fitness does not either.  Below a million first-layer products a
 // spark (64-32-10, N = 300, 64 sparks: 19 us there, 22 us here) a launch is
 // bound by its fixed latency, which is longer here; under 16 inputs or 8
-// hidden units most of a block or a tile would be padding.
+// hidden units most of a block or a tile would be padding.  Above, the first
+// layer is far faster here and the later layers are slower: one warp to a
+// spark's 32 samples, a tile's spare columns idle, 25 classes and more in
+// registers that spill.  So a tile's estimated times are compared: here the
+// splitting or, where it is longer, the layers after it.  The estimates were
+// fitted to 998 timed launches of 40 to 1,040 sparks (16 <= d_in <= 3072, 8 <=
+// h1 <= 128, h2 <= 64, 2 to 32 classes; 5% off here, 9% there); of 3,587 such
+// and smaller launches, us there / here: 784-64-10 (N = 84, 1,040 sparks) 420 /
+// 120, 256-64-32 (512, 333) 182 / 157, 64-64-32 (2048, 333) 373 / 473,
+// 16-8-64-32 (8192, 1,040) 7,232 / 16,761, 16-43-24-5 (3049, 1,040) 1,173 / 2,476.
 constexpr int kMinInputs = 16, kMinHidden = 8;
 constexpr int64_t kMinProducts = int64_t(1) << 20;
+
+// Nanoseconds of a tile on one SM, V sparks to a tile.
+int64_t tile_ns(const Mlp& mlp, int V) {
+  const int L = mlp.n_layers, h1 = mlp.widths[1], h2 = L == 3 ? mlp.widths[2] : 0, C = mlp.widths[L];
+  const bool v4 = h1 % 4 == 0 && h2 % 4 == 0;
+  // a spark's logits, per input of the last layer: by the register slots, 16-byte weight reads or not
+  const int slots = C <= 4 ? 0 : C <= 10 ? 1 : C <= 16 ? 2 : C <= 24 ? 3 : 4;
+  constexpr int kLogit[2][5] = {{40, 77, 159, 302, 660}, {19, 46, 81, 141, 507}}, kSlots[5] = {4, 10, 16, 24, 32};
+  const int64_t rounds10 = V > 1 ? 5 * V : 7;  // eight (spark, 32 samples) items to a round; four alone take 0.7
+  int64_t tail = 4200 + (mlp.acts[0] == kActTanh ? 1100 : 0) +
+                 rounds10 * (kLogit[v4][slots] * mlp.widths[L - 1] + 66 * kSlots[slots]) / 10;
+  if (L == 3) {
+    const int units = (h2 + 7) / 8 * V;
+    tail += (C > 10 ? 7200 : 5000) + (int64_t)h1 * (v4 ? 15 + 20 * units : 54 + 62 * units);
+  }
+  const int64_t split = (int64_t)(mlp.widths[0] + kKB - 1) / kKB * 940;
+  const int64_t after = tail + (split > 1100 ? split - 1100 : 0);  // the next tile's first block is split meanwhile
+  return split > after ? split : after;
+}
 
 bool fitness_x3_ok(const Mlp& mlp) {
   if (mlp.widths[0] % 8 != 0 || mlp.widths[0] < kMinInputs || mlp.widths[1] < kMinHidden || mlp.widths[1] > kN ||
       mlp.w1_elems * mlp.N < kMinProducts || (mlp.n_layers == 3 && mlp.widths[2] > 8 * kEpiWarps))
     return false;
-  return smem_for(mlp, 1, kMaxStages - 1) <= kSmemLimit;
+  const int V = sparks_per_tile(mlp);
+  return smem_for(mlp, 1, kMaxStages - 1) <= kSmemLimit && 97 * tile_ns(mlp, V) <= 100 * V * fitness_simt_ns(mlp);
 }
 
 int launch_fitness_x3(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial, uint32_t* status,

@@ -313,6 +313,7 @@ int launch_select(const Problem& p, const float* fit_e, float* fit_g, const floa
 int launch_fitness_fp32(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial,
                         uint32_t* status, uint64_t wait_budget, cudaStream_t s);
 bool fitness_x3_ok(const Mlp& mlp);
+int64_t fitness_simt_ns(const Mlp& mlp);
 int launch_fitness_x3(const Mlp& mlp, const float* rows, int64_t ld, int32_t count, float* partial, uint32_t* status,
                       uint64_t wait_budget, cudaStream_t s);
 
