@@ -194,9 +194,13 @@ struct SmallNet {
 // GPU (200 and 20 sparks x 512 samples with eight per block: 14.3 us a
 // launch either way; with one, whole generations went from 91 to 30 us).
 constexpr int kSmallSparks = 8;
+// Blocks per SM that the registers must allow, 40 a thread.  Left to itself the compiler takes 32, whose order of the
+// chains costs a small launch 1 us of 4 (a run of 90 generations 2,855 us, 2,670 so); 64 gain as much again there but
+// lose 2% where the blocks fill the GPU (N = 131,072, 200 sparks: 94.7 us, 93.9 so).
+constexpr int kSmallBlocks = 12;
 
 template <int DI, int H1, int C>
-__global__ void __launch_bounds__(kMT) k_fitness_small(Mlp mlp, const float* __restrict__ rows, int64_t ld,
+__global__ void __launch_bounds__(kMT, kSmallBlocks) k_fitness_small(Mlp mlp, const float* __restrict__ rows, int64_t ld,
                                                        int32_t count, int32_t per, float* __restrict__ partial) {
   using Net = SmallNet<DI, H1, C>;
   __shared__ float ws[kSmallSparks][Net::D];
@@ -205,9 +209,11 @@ __global__ void __launch_bounds__(kMT) k_fitness_small(Mlp mlp, const float* __r
   griddep_launch_dependents();
   const int s0 = blockIdx.x * per, mt = blockIdx.y;
   const int gs = min(per, count - s0);
-  for (int e = threadIdx.x; e < gs * Net::D; e += kMT) {
-    const int g = e / Net::D, k = e - g * Net::D;
-    ws[g][k] = rows[(int64_t)(s0 + g) * ld + k];
+  for (int g = 0; g < gs; ++g) {
+    const float* row = rows + (int64_t)(s0 + g) * ld;
+#pragma unroll
+    for (int k0 = 0; k0 < Net::D; k0 += kMT)
+      if (k0 + (int)threadIdx.x < Net::D) ws[g][k0 + threadIdx.x] = row[k0 + threadIdx.x];
   }
   const int64_t n = (int64_t)mt * kMT + threadIdx.x;
   const bool valid = n < mlp.N;
