@@ -485,7 +485,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_fitness_x3(const __grid_constan
       if (redo != 0) {
         // those columns of this sample again, in FP32 in index order; a NaN among the inputs needs no more looking,
         // and a sum that has become one stays it (784-64-10, N = 2048, 1,000 sparks, one input NaN in every sample:
-        // 4.2 ms, all chains to their end 225, k_fitness_simt 6.0, finite inputs 1.6)
+        // 4.2 ms, all chains to their end 225, k_fitness_simt 6.0, finite inputs 1.6; an infinite input in every sample,
+        // X read from L2 once a column, 150)
         const float* xr = mlp.X + n * d_in;
         float x_nan = 0.0f;
 #pragma unroll 1
