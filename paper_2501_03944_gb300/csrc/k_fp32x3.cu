@@ -741,6 +741,9 @@ __device__ __forceinline__ void net_store8(const NetX3Args& a, int64_t r, int co
   }
 }
 
+// kBudget: the waits' limit is a.wait_budget, else the default (with it always read from the argument a run of the
+// 1000-512x11-1 network took 0.9% longer).
+template <bool kBudget>
 __global__ void __launch_bounds__(kNetThreads, 1)
     k_net_x3(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w, NetX3Args a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -759,6 +762,7 @@ __global__ void __launch_bounds__(kNetThreads, 1)
   const int sp0 = (int)blockIdx.z * a.per, nsp = min(a.per, a.splits - sp0);
   const int kb0 = sp0 * kNetKPer;
   const int nkb = min(nsp * kNetKPer, a.k_blocks - kb0);
+  auto budget = [&] { return kBudget ? a.wait_budget : kWaitBudget; };
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&sb->full[s], 1);
@@ -807,7 +811,7 @@ __global__ void __launch_bounds__(kNetThreads, 1)
       for (int kb = 0; kb < first; ++kb) load_a(kb);
       int kb = first;
       for (; kb < nkb; ++kb) {
-        if (!mbar_wait(sb, &sb->empty[kb % S], (uint32_t)(kb / S - 1) & 1u, a.status, 1u, a.wait_budget)) break;
+        if (!mbar_wait(sb, &sb->empty[kb % S], (uint32_t)(kb / S - 1) & 1u, a.status, 1u, budget())) break;
         mbar_expect_tx(&sb->full[kb % S], kStageBytes);
         load_w(kb);
         load_a(kb);
@@ -822,11 +826,11 @@ __global__ void __launch_bounds__(kNetThreads, 1)
       bool ok = true;
       for (int i = 0; i < nsp; ++i) {
         // the accumulators are free once the epilogue has read the split before
-        if (ok && i > 0) ok = mbar_wait(sb, &sb->read, (uint32_t)(i - 1) & 1u, a.status, 4u, a.wait_budget);
+        if (ok && i > 0) ok = mbar_wait(sb, &sb->read, (uint32_t)(i - 1) & 1u, a.status, 4u, budget());
         const int k1 = min((i + 1) * kNetKPer, nkb);
         for (int kb = i * kNetKPer; ok && kb < k1; ++kb) {
           const int s = kb % S, l = kb - i * kNetKPer;  // l: block of the split
-          if (!mbar_wait(sb, &sb->full[s], (uint32_t)(kb / S) & 1u, a.status, 2u, a.wait_budget)) {
+          if (!mbar_wait(sb, &sb->full[s], (uint32_t)(kb / S) & 1u, a.status, 2u, budget())) {
             ok = false;
             break;
           }
@@ -1058,7 +1062,8 @@ bool net_x3_plan(NetX3Plan& pl, const NetOut& net, int64_t max_rows, uint32_t* b
       if (!encode_bf16(&pl.tmap_w[l], pl.w_parts[l], dims, strides, box)) return false;
     }
   }
-  if (!any || ensure_smem_limit<k_net_x3>(net_x3_smem(2)) != cudaSuccess) {
+  if (!any || ensure_smem_limit<k_net_x3<false>>(net_x3_smem(2)) != cudaSuccess ||
+      ensure_smem_limit<k_net_x3<true>>(net_x3_smem(2)) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -1118,11 +1123,12 @@ int launch_net_output_x3(const NetX3Plan& pl, const NetOut& net, const float* ro
       x.parts = next_tc ? pl.act_parts[(l + 1) & 1] : nullptr;
       x.plane_words = pl.max_rows * (fo / 2);
       x.status = status;
-      x.wait_budget = pl.wait_budget != 0 ? pl.wait_budget : kWaitBudget;
+      x.wait_budget = pl.wait_budget;
       const dim3 grid((unsigned)((count + kBM - 1) / kBM), (unsigned)((fo + kN - 1) / kN),
                       (unsigned)((x.splits + x.per - 1) / x.per));
-      if (launch_pdl_z(k_net_x3, grid, dim3(kNetThreads), net_x3_smem(x.per), x.partial ? 1u : grid.z, s,
-                       pl.tmap_a[l], pl.tmap_w[l], x) != cudaSuccess)
+      if (launch_pdl_z(pl.wait_budget != 0 ? k_net_x3<true> : k_net_x3<false>, grid, dim3(kNetThreads),
+                       net_x3_smem(x.per), x.partial ? 1u : grid.z, s, pl.tmap_a[l], pl.tmap_w[l],
+                       x) != cudaSuccess)
         return -1;
       ++n;
       if (x.partial) {
